@@ -420,8 +420,8 @@ int amr_mlp_train(int dim, const float* X, const float* y, long n, float pos_wei
  * X (n x K floats), y (n floats), weights (flat layout of amr_set_mlp), grad
  * (same layout, output) and loss (one float, output) are DEVICE pointers owned
  * by the caller; work is issued on `stream` (a cudaStream_t, NULL = legacy
- * stream) and not synchronised. The hidden activations use a fixed scratch
- * array compiled into the library (about 2.1 MB on every GPU that loads it,
+ * stream) and not synchronised. The passes between the kernels use a fixed scratch
+ * array compiled into the library (about 1.7 MB on every GPU that loads it,
  * held until the process exits), so n is limited to
  * AMR_MLP_NOALLOC_MAX_ROWS; larger n returns AMR_ERR_ARG. The call allocates
  * nothing. Its first call on a device looks up the array's device address

@@ -3,6 +3,7 @@
 // training. The paper leaves the refinement criterion to the runtime program
 // (Sec. 4.2); this network is one such program. Training is deterministic:
 // every reduction is a fixed-order loop, no atomics.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,6 +26,7 @@ long mlp_n_weights(int dim) {
 }  // namespace amr
 
 using namespace amr;
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -119,85 +121,315 @@ __global__ void __launch_bounds__(512, 1) k_infer(const float* __restrict__ X, l
 }
 
 // ---------------------------------------------------------------------------
-// FP32 training kernels (rows of a minibatch selected by idx)
+// FP32 training kernels (rows of a minibatch selected by idx): loss and
+// gradient of n rows in three launches.
+//   k_rows     everything that is local to a row: both hidden layers, the
+//              logit, dz, the gradients of the hidden layers, and this block's
+//              part of the gradients of b1, W2, b2, w3, b3 and of the loss
+//   k_w1grad   dW1 = dH1^T X, split over the rows
+//   k_gradsum  the parts added in a fixed order (and the Adam update in training)
+// Every sum has a fixed order, so equal calls give equal bits.
 // ---------------------------------------------------------------------------
-__global__ void k_dense_relu(const float* __restrict__ In, const int* __restrict__ idx, int n, int I,
-                             const float* __restrict__ W, const float* __restrict__ b, float* __restrict__ H) {
-    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t >= (long)n * MLP_H) return;
-    const int r = (int)(t / MLP_H), o = (int)(t % MLP_H);
-    const float* x = In + (long)(idx ? idx[r] : r) * I;
-    const float* wr = W + (long)o * I;
-    float acc = b[o];
-    for (int k = 0; k < I; ++k) acc += x[k] * wr[k];
-    H[t] = fmaxf(acc, 0.f);
-}
-
 __device__ __forceinline__ float softplus(float x) { return fmaxf(x, 0.f) + log1pf(expf(-fabsf(x))); }
 
-__global__ void k_out(const float* __restrict__ H2, int n, const float* __restrict__ w3, const float* __restrict__ b3,
-                      const float* __restrict__ y, const int* __restrict__ idx, float pw, float* __restrict__ dz,
-                      float* __restrict__ lossv) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    float z = b3[0];
-    for (int j = 0; j < MLP_H; ++j) z += H2[(long)r * MLP_H + j] * w3[j];
-    const float yy = y[idx ? idx[r] : r];
-    const float sg = 0.5f * (1.f + tanhf(0.5f * z));
-    lossv[r] = pw * yy * softplus(-z) + (1.f - yy) * softplus(z);
-    dz[r] = (pw * yy * (sg - 1.f) + (1.f - yy) * sg) / (float)n;
+// the gradients of b1, W2, b2, w3, b3 (the flat layout after W1), then the loss
+constexpr int SMALL = MLP_H + MLP_H * MLP_H + MLP_H + MLP_H + 1;
+constexpr int SMALL_L = SMALL + 1;
+constexpr int ROWS_NTH = 512;
+constexpr int ROWS_CL = 4;                  // blocks of a cluster, whose parts are added in shared memory
+constexpr int ROWS_MAXCL = 32;              // clusters of a launch
+constexpr int W1_CT = 16;                   // columns of X of a k_w1grad block
+constexpr int W1_RC = 64;                   // rows staged at a time
+constexpr int W1_PARTS = 160000;            // floats of the split dW1 (4 x 64 x 625)
+
+// row splits of k_w1grad: about one block per SM over the column tiles, as far
+// as the parts fit their buffer
+__host__ __device__ constexpr int w1_tiles(int K) { return (K + W1_CT - 1) / W1_CT; }
+__host__ __device__ constexpr int w1_splits(int K) {
+    int s = 160 / w1_tiles(K);
+    const int fit = W1_PARTS / (MLP_H * K);
+    s = s < fit ? s : fit;
+    return s < 32 ? s : 32;
 }
 
-// dH = (dOut @ W) * (H > 0); dOut (n x O), W (O x 64)
-__global__ void k_back_hidden(const float* __restrict__ dOut, int n, int O, const float* __restrict__ W,
-                              const float* __restrict__ H, float* __restrict__ dH) {
-    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t >= (long)n * MLP_H) return;
-    const int r = (int)(t / MLP_H), j = (int)(t % MLP_H);
-    float acc = 0.f;
-    for (int o = 0; o < O; ++o) acc += dOut[(long)r * O + o] * W[(long)o * MLP_H + j];
-    dH[t] = H[t] > 0.f ? acc : 0.f;
-}
-
-// dW[o][i] = sum_r dOut[r][o] In[row(r)][i]  (i < I), db[o] = sum_r dOut[r][o]
-__global__ void k_wgrad(const float* __restrict__ dOut, int n, int O, const float* __restrict__ In,
-                        const int* __restrict__ idx, int I, float* __restrict__ dW, float* __restrict__ db) {
-    const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (t >= (long)O * (I + 1)) return;
-    const int o = (int)(t / (I + 1)), i = (int)(t % (I + 1));
-    float acc = 0.f;
-    if (i < I) {
-        for (int r = 0; r < n; ++r) acc += dOut[(long)r * O + o] * In[(long)(idx ? idx[r] : r) * I + i];
-        dW[(long)o * I + i] = acc;
-    } else {
-        for (int r = 0; r < n; ++r) acc += dOut[(long)r * O + o];
-        db[o] = acc;
+// Sums v[0 .. M) over the 32 lanes: at each step a lane keeps the half of its
+// values that its lane bit names and adds the partner's, so the whole sum
+// takes M - 1 (+ the steps left once one value remains) shuffles instead of
+// 5 M. Afterwards lane holds the values `base ..`, max(M / 32, 1) of them.
+template <int M>
+__device__ __forceinline__ int lane_sums(float (&v)[M]) {
+    const int lane = threadIdx.x & 31;
+    int base = 0, m = M;
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) {
+        if (m > 1) {
+            m >>= 1;
+            const bool hi = lane & s;
+            if (hi) base += m;
+#pragma unroll
+            for (int i = 0; i < M / 2; ++i) {
+                if (i < m) {
+                    const float keep = hi ? v[i + m] : v[i], send = hi ? v[i] : v[i + m];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+                }
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], s);
+        }
     }
+    return base;
 }
 
-__global__ void k_sum(const float* __restrict__ v, int n, float* __restrict__ out, float scale) {
-    __shared__ float red[256];
-    float acc = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) acc += v[i];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+// R rows per tile. Layer 1 is the work: a warp owns 4 of the 64 outputs, its
+// lanes run along K (W1 is read once per block, coalesced, from L2, the rows
+// from shared memory), and the lanes' sums are added at the end. Bound by the
+// L2 latency of the W1 stream and FMA issue. The three launches take 42 us for
+// the 3D gradient of 2048 rows; with one thread per (row, output) or weight,
+// each looping serially over K or over all the rows, it took 772 us.
+template <int D, int R>
+__global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
+    k_rows(const float* __restrict__ X, const int* __restrict__ idx, const float* __restrict__ y, long n, float pw,
+           const float* __restrict__ w, float* __restrict__ dH1, float* __restrict__ part) {
+    constexpr int K = mlp_kin(D), H = MLP_H, P2 = H + 1;
+    constexpr int KS = (K + 31) / 32, OW = H / (ROWS_NTH / 32);     // lane steps; outputs per warp
+    constexpr int AREA0 = R * K > H * P2 + R * H ? R * K : H * P2 + R * H;
+    constexpr int AREA = AREA0 > SMALL_L ? AREA0 : SMALL_L;
+    // the rows of X, later W2 (padded rows) and dH1, at the end the block's sums
+    __shared__ float area[AREA];
+    __shared__ float H1[R * H], H2[R * H];
+    __shared__ float dz[R], ls[R];
+    float* Xs = area;
+    float* W2s = area;
+    float* D1 = area + H * P2;
+    const float* W1 = w;
+    const float* b1 = W1 + H * K;
+    const float* W2 = b1 + H;
+    const float* b2 = W2 + H * H;
+    const float* w3 = b2 + H;
+    const float* b3 = w3 + H;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int o = t & (H - 1), rg = t >> 6;                // (output, row group) of the small products
+    float aw2[H * H / ROWS_NTH], as = 0.f;                 // this thread's entries of dW2; of the vectors
+#pragma unroll
+    for (int i = 0; i < H * H / ROWS_NTH; ++i) aw2[i] = 0.f;
+    const long tiles = (n + R - 1) / R;
+    for (long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const long r0 = tile * R;
+        const int nr = (int)(n - r0 < R ? n - r0 : R);
+        for (int i = t; i < R * K; i += ROWS_NTH) {
+            const int r = i / K, k = i - r * K;
+            Xs[i] = r < nr ? X[(long)(idx ? idx[r0 + r] : r0 + r) * K + k] : 0.f;
+        }
+        __syncthreads();
+        {
+            float acc[OW * R];
+#pragma unroll
+            for (int i = 0; i < OW * R; ++i) acc[i] = 0.f;
+#pragma unroll 4
+            for (int ks = 0; ks < KS; ++ks) {
+                const int k = ks * 32 + lane;
+                const int kk = k < K ? k : K - 1;
+                float wv[OW];
+#pragma unroll
+                for (int j = 0; j < OW; ++j) {
+                    const float x = W1[(warp * OW + j) * K + kk];
+                    wv[j] = k < K ? x : 0.f;
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float x = Xs[r * K + kk];
+#pragma unroll
+                    for (int j = 0; j < OW; ++j) acc[j * R + r] = fmaf(x, wv[j], acc[j * R + r]);
+                }
+            }
+            const int base = lane_sums<OW * R>(acc);
+            constexpr int LEFT = OW * R >= 32 ? OW * R / 32 : 1;
+#pragma unroll
+            for (int i = 0; i < LEFT; ++i) {
+                const int j = (base + i) / R, r = (base + i) % R, oo = warp * OW + j;
+                H1[r * H + oo] = fmaxf(acc[i] + b1[oo], 0.f);
+            }
+        }
+        __syncthreads();                                   // the rows of X are read; H1 is written
+        for (int i = t; i < H * H; i += ROWS_NTH) W2s[(i >> 6) * P2 + (i & (H - 1))] = W2[i];
+        __syncthreads();
+        for (int r = rg; r < R; r += ROWS_NTH / H) {
+            float acc = b2[o];
+#pragma unroll 16
+            for (int k = 0; k < H; ++k) acc = fmaf(H1[r * H + k], W2s[o * P2 + k], acc);
+            H2[r * H + o] = fmaxf(acc, 0.f);
+        }
+        __syncthreads();
+        if (warp < R) {
+            float z = H2[warp * H + lane] * w3[lane] + H2[warp * H + lane + 32] * w3[lane + 32];
+#pragma unroll
+            for (int s = 16; s >= 1; s >>= 1) z += __shfl_xor_sync(0xffffffffu, z, s);
+            if (lane == 0) {
+                z += b3[0];
+                float d = 0.f, l = 0.f;
+                if (warp < nr) {
+                    const float yy = y[idx ? idx[r0 + warp] : r0 + warp];
+                    const float sg = 0.5f * (1.f + tanhf(0.5f * z));
+                    l = pw * yy * softplus(-z) + (1.f - yy) * softplus(z);
+                    d = (pw * yy * (sg - 1.f) + (1.f - yy) * sg) / (float)n;
+                }
+                dz[warp] = d;
+                ls[warp] = l;
+            }
+        }
+        __syncthreads();
+        if (t >= 128 && t < 192) {                         // dw3
+            for (int r = 0; r < R; ++r) as = fmaf(dz[r], H2[r * H + t - 128], as);
+        } else if (t == 192) {
+            for (int r = 0; r < R; ++r) as += dz[r];
+        } else if (t == 193) {
+            for (int r = 0; r < R; ++r) as += ls[r];
+        }
+        __syncthreads();
+        for (int r = rg; r < R; r += ROWS_NTH / H) H2[r * H + o] = H2[r * H + o] > 0.f ? dz[r] * w3[o] : 0.f;   // dH2
+        __syncthreads();
+        for (int r = rg; r < R; r += ROWS_NTH / H) {
+            float acc = 0.f;
+#pragma unroll 16
+            for (int q = 0; q < H; ++q) acc = fmaf(H2[r * H + q], W2s[q * P2 + o], acc);
+            const float d = H1[r * H + o] > 0.f ? acc : 0.f;
+            D1[r * H + o] = d;
+            if (r < nr) dH1[(r0 + r) * H + o] = d;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float d = H2[r * H + (t >> 3)];
+#pragma unroll
+            for (int i = 0; i < H * H / ROWS_NTH; ++i) aw2[i] = fmaf(d, H1[r * H + (t & 7) + 8 * i], aw2[i]);
+        }
+        __syncthreads();
+        if (t < 64) {
+            for (int r = 0; r < R; ++r) as += D1[r * H + t];
+        } else if (t < 128) {
+            for (int r = 0; r < R; ++r) as += H2[r * H + t - 64];
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[0] += red[0] * scale;
+    // the block's part, then the cluster's
+    if (t < 64) area[t] = as;
+    else if (t < 194) area[H * H + t] = as;                // b2, w3, b3, loss follow W2
+#pragma unroll
+    for (int i = 0; i < H * H / ROWS_NTH; ++i) area[H + (t >> 3) * H + (t & 7) + 8 * i] = aw2[i];
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    const int rank = (int)cl.block_rank();
+    for (int e = rank * ROWS_NTH + t; e < SMALL_L; e += ROWS_CL * ROWS_NTH) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < ROWS_CL; ++q) s += *cl.map_shared_rank(area + e, q);
+        part[(long)(blockIdx.x / ROWS_CL) * SMALL_L + e] = s;
+    }
+    cl.sync();                                             // a block's sums stay until its peers have read them
 }
 
-__global__ void k_adam(float* __restrict__ w, const float* __restrict__ gr, float* __restrict__ m,
-                       float* __restrict__ v, long n, float lr, float c1, float c2) {
-    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float g = gr[i];
-    const float mi = 0.9f * m[i] + 0.1f * g;
-    const float vi = 0.999f * v[i] + 0.001f * g * g;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+// dW1 of W1_CT columns over one split of the rows: rows are staged 64 at a time
+// (the next ones on their way in registers), a thread owns 8 outputs x 2
+// columns and every fourth row, so that 16 FMAs share three shared-memory
+// loads; the four row groups are added in order at the end. FMA issue bound.
+template <int D>
+__global__ void __launch_bounds__(256) k_w1grad(const float* __restrict__ dH1, const float* __restrict__ X,
+                                                const int* __restrict__ idx, long n, float* __restrict__ part) {
+    constexpr int K = mlp_kin(D), H = MLP_H, CT = W1_CT, RC = W1_RC;
+    constexpr int ND = RC * H / 4 / 256, NX = RC * CT / 256;
+    __shared__ __align__(16) float ds[RC * H];
+    __shared__ __align__(16) float xs[RC * CT];
+    static_assert(4 * H * CT <= RC * H, "the row groups' sums fit the staged rows");
+    const int t = threadIdx.x, k0 = blockIdx.x * CT;
+    const long per = (n + gridDim.y - 1) / gridDim.y;
+    const long lo = blockIdx.y * per, hi = lo + per < n ? lo + per : n;
+    float4 rd[ND];
+    float rx[NX];
+    auto fetch = [&](long b) {
+#pragma unroll
+        for (int i = 0; i < ND; ++i) {
+            const int e = t + i * 256;
+            const long r = b + (e >> 4);
+            rd[i] = r < hi ? *reinterpret_cast<const float4*>(dH1 + r * H + (e & 15) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < NX; ++i) {
+            const int e = t + i * 256, k = k0 + (e & (CT - 1));
+            const long r = b + e / CT;
+            rx[i] = (r < hi && k < K) ? X[(long)(idx ? idx[r] : r) * K + k] : 0.f;
+        }
+    };
+    const int g = t >> 6, og = (t & 63) >> 3, kg = t & 7;   // row group, 8 outputs, 2 columns
+    float acc[8][2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = 0.f;
+    fetch(lo);
+    for (long b = lo; b < hi; b += RC) {
+#pragma unroll
+        for (int i = 0; i < ND; ++i) reinterpret_cast<float4*>(ds)[t + i * 256] = rd[i];
+#pragma unroll
+        for (int i = 0; i < NX; ++i) xs[t + i * 256] = rx[i];
+        __syncthreads();
+        if (b + RC < hi) fetch(b + RC);
+#pragma unroll 4
+        for (int r = g; r < RC; r += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(ds + r * H + og * 8);
+            const float4 c = *reinterpret_cast<const float4*>(ds + r * H + og * 8 + 4);
+            const float2 x = *reinterpret_cast<const float2*>(xs + r * CT + kg * 2);
+            const float d[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                acc[i][0] = fmaf(d[i], x.x, acc[i][0]);
+                acc[i][1] = fmaf(d[i], x.y, acc[i][1]);
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        ds[(g * H + og * 8 + i) * CT + kg * 2] = acc[i][0];
+        ds[(g * H + og * 8 + i) * CT + kg * 2 + 1] = acc[i][1];
+    }
+    __syncthreads();
+    for (int e = t; e < H * CT; e += 256) {
+        const int k = k0 + (e & (CT - 1));
+        if (k < K)
+            part[((long)blockIdx.y * H + e / CT) * K + k] = ((ds[e] + ds[H * CT + e]) + ds[2 * H * CT + e]) + ds[3 * H * CT + e];
+    }
+}
+
+struct AdamStep {
+    float* w;               // nullptr: gradient only
+    float* m;
+    float* v;
+    float lr, c1, c2;
+};
+
+// One thread per weight adds its parts in order; the thread past the weights
+// adds the loss (scaled; onto *loss where `add`).
+__global__ void __launch_bounds__(256) k_gradsum(int K, const float* __restrict__ p1, int s1,
+                                                 const float* __restrict__ p2, int s2, float* __restrict__ gr,
+                                                 float* loss, float scale, int add, AdamStep a) {
+    const int n1 = MLP_H * K;
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= n1 + SMALL_L) return;
+    const bool first = i < n1;
+    const float* p = first ? p1 + i : p2 + (i - n1);
+    const int cnt = first ? s1 : s2, step = first ? n1 : SMALL_L;
+    float g = 0.f;
+#pragma unroll 8
+    for (int q = 0; q < cnt; ++q) g += p[(long)q * step];
+    if (i == n1 + SMALL) {
+        if (loss) loss[0] = add ? loss[0] + g * scale : g * scale;
+        return;
+    }
+    if (gr) gr[i] = g;
+    if (a.w) {
+        const float mi = 0.9f * a.m[i] + 0.1f * g;
+        const float vi = 0.999f * a.v[i] + 0.001f * g * g;
+        a.m[i] = mi;
+        a.v[i] = vi;
+        a.w[i] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + 1e-8f);
+    }
 }
 
 // minibatch rows of an epoch: an affine permutation r -> (a r + b) mod n
@@ -229,34 +461,49 @@ cudaStream_t stream_of(const amr_options_t* o) { return o ? reinterpret_cast<cud
 
 int blocks(long n, int b = 256) { return (int)((n + b - 1) / b); }
 
-// one forward + backward pass over `n` rows; gradient to g (flat layout)
-int fwd_bwd(int D, const float* X, const int* idx, const float* y, int n, float pw, const float* w, float* g,
-            float* loss_acc, float loss_scale, float* H1, float* H2, float* dz, float* lossv, float* dH1, float* dH2,
-            cudaStream_t s) {
-    const int K = mlp_kin(D);
-    const float* W1 = w;
-    const float* b1 = W1 + MLP_H * K;
-    const float* W2 = b1 + MLP_H;
-    const float* b2 = W2 + MLP_H * MLP_H;
-    const float* w3 = b2 + MLP_H;
-    const float* b3 = w3 + MLP_H;
-    float* gW1 = g;
-    float* gb1 = gW1 + MLP_H * K;
-    float* gW2 = gb1 + MLP_H;
-    float* gb2 = gW2 + MLP_H * MLP_H;
-    float* gw3 = gb2 + MLP_H;
-    float* gb3 = gw3 + MLP_H;
-    const long nh = (long)n * MLP_H;
-    k_dense_relu<<<blocks(nh), 256, 0, s>>>(X, idx, n, K, W1, b1, H1);
-    k_dense_relu<<<blocks(nh), 256, 0, s>>>(H1, nullptr, n, MLP_H, W2, b2, H2);
-    k_out<<<blocks(n), 256, 0, s>>>(H2, n, w3, b3, y, idx, pw, dz, lossv);
-    k_wgrad<<<blocks(MLP_H + 1), 256, 0, s>>>(dz, n, 1, H2, nullptr, MLP_H, gw3, gb3);
-    k_back_hidden<<<blocks(nh), 256, 0, s>>>(dz, n, 1, w3, H2, dH2);
-    k_wgrad<<<blocks((long)MLP_H * (MLP_H + 1)), 256, 0, s>>>(dH2, n, MLP_H, H1, nullptr, MLP_H, gW2, gb2);
-    k_back_hidden<<<blocks(nh), 256, 0, s>>>(dH2, n, MLP_H, W2, H1, dH1);
-    k_wgrad<<<blocks((long)MLP_H * (K + 1)), 256, 0, s>>>(dH1, n, MLP_H, X, idx, K, gW1, gb1);
-    if (loss_acc) k_sum<<<1, 256, 0, s>>>(lossv, n, loss_acc, loss_scale);
+// Scratch of a gradient over n rows, in floats: dH1, the clusters' parts of
+// k_rows, the splits' parts of k_w1grad
+struct GradScratch {
+    float *dH1, *small, *w1;
+    static constexpr size_t SMALL_PARTS = (size_t)ROWS_MAXCL * SMALL_L;
+    static constexpr size_t floats(long n) { return ((size_t)n * MLP_H + 3) / 4 * 4 + SMALL_PARTS + W1_PARTS; }
+    GradScratch(float* base, long n) {
+        dH1 = base;
+        small = base + ((size_t)n * MLP_H + 3) / 4 * 4;
+        w1 = small + SMALL_PARTS;
+    }
+};
+
+// one forward + backward pass over `n` rows; gradient to g (flat layout; may
+// be null), loss times loss_scale to *loss (added to it where `add`; may be null)
+template <int D>
+int fwd_bwd_d(const float* X, const int* idx, const float* y, long n, float pw, const float* w, float* g, float* loss,
+              float loss_scale, int add, const GradScratch& sc, const AdamStep& adam, cudaStream_t s) {
+    constexpr int K = mlp_kin(D);
+    static_assert(w1_splits(K) >= 1 && w1_splits(K) * MLP_H * K <= W1_PARTS, "the parts fit");
+    // rows per tile: the fewest that a launch of 128 blocks covers in one pass
+    // (a block's time is its W1 stream, then its rows); 16 beyond
+    const int R = n <= 4 * ROWS_CL * ROWS_MAXCL ? 4 : (n <= 8 * ROWS_CL * ROWS_MAXCL ? 8 : 16);
+    const long tiles = (n + R - 1) / R;
+    const int ncl = (int)std::min<long>((tiles + ROWS_CL - 1) / ROWS_CL, ROWS_MAXCL);
+    const int grid = ncl * ROWS_CL;
+    if (R == 4) k_rows<D, 4><<<grid, ROWS_NTH, 0, s>>>(X, idx, y, n, pw, w, sc.dH1, sc.small);
+    else if (R == 8) k_rows<D, 8><<<grid, ROWS_NTH, 0, s>>>(X, idx, y, n, pw, w, sc.dH1, sc.small);
+    else k_rows<D, 16><<<grid, ROWS_NTH, 0, s>>>(X, idx, y, n, pw, w, sc.dH1, sc.small);
+    const int splits = (int)std::min<long>(w1_splits(K), (n + W1_RC - 1) / W1_RC);
+    k_w1grad<D><<<dim3(w1_tiles(K), splits), 256, 0, s>>>(sc.dH1, X, idx, n, sc.w1);
+    k_gradsum<<<(MLP_H * K + SMALL_L + 255) / 256, 256, 0, s>>>(K, sc.w1, splits, sc.small, ncl, g, loss, loss_scale,
+                                                                add, adam);
     return cudaGetLastError() == cudaSuccess ? AMR_OK : AMR_ERR_CUDA;
+}
+
+int fwd_bwd(int D, const float* X, const int* idx, const float* y, long n, float pw, const float* w, float* g,
+            float* loss, float loss_scale, int add, const GradScratch& sc, const AdamStep& adam, cudaStream_t s) {
+    switch (D) {
+    case 1: return fwd_bwd_d<1>(X, idx, y, n, pw, w, g, loss, loss_scale, add, sc, adam, s);
+    case 2: return fwd_bwd_d<2>(X, idx, y, n, pw, w, g, loss, loss_scale, add, sc, adam, s);
+    default: return fwd_bwd_d<3>(X, idx, y, n, pw, w, g, loss, loss_scale, add, sc, adam, s);
+    }
 }
 
 template <int D>
@@ -332,19 +579,13 @@ int amr_mlp_grad(int dim, const float* X, const float* y, long n, float pw, cons
     float* dy = dv.get<float>(n);
     float* dw = dv.get<float>(nw);
     float* dg = dv.get<float>(nw);
-    float* H1 = dv.get<float>(n * MLP_H);
-    float* H2 = dv.get<float>(n * MLP_H);
-    float* dH1 = dv.get<float>(n * MLP_H);
-    float* dH2 = dv.get<float>(n * MLP_H);
-    float* dz = dv.get<float>(n);
-    float* lv = dv.get<float>(n);
+    float* scr = dv.get<float>(GradScratch::floats(n));
     float* la = dv.get<float>(1);
-    if (!dx || !dy || !dw || !dg || !H1 || !H2 || !dH1 || !dH2 || !dz || !lv || !la) return AMR_ERR_CUDA;
+    if (!dx || !dy || !dw || !dg || !scr || !la) return AMR_ERR_CUDA;
     cudaMemcpyAsync(dx, X, n * K * sizeof(float), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(dy, y, n * sizeof(float), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(dw, weights, nw * sizeof(float), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(la, 0, sizeof(float), s);
-    if (fwd_bwd(dim, dx, nullptr, dy, (int)n, pw, dw, dg, la, 1.0f / (float)n, H1, H2, dz, lv, dH1, dH2, s))
+    if (fwd_bwd(dim, dx, nullptr, dy, n, pw, dw, dg, la, 1.0f / (float)n, 0, GradScratch(scr, n), AdamStep{}, s))
         return AMR_ERR_CUDA;
     cudaMemcpyAsync(grad, dg, nw * sizeof(float), cudaMemcpyDeviceToHost, s);
     if (loss) cudaMemcpyAsync(loss, la, sizeof(float), cudaMemcpyDeviceToHost, s);
@@ -363,19 +604,13 @@ int amr_mlp_train(int dim, const float* X, const float* y, long n, float pw, int
     float* dx = dv.get<float>(n * K);
     float* dy = dv.get<float>(n);
     float* dw = dv.get<float>(nw);
-    float* dg = dv.get<float>(nw);
     float* m = dv.get<float>(nw);
     float* v = dv.get<float>(nw);
     int* idx = dv.get<int>(n);
-    float* H1 = dv.get<float>((long)B * MLP_H);
-    float* H2 = dv.get<float>((long)B * MLP_H);
-    float* dH1 = dv.get<float>((long)B * MLP_H);
-    float* dH2 = dv.get<float>((long)B * MLP_H);
-    float* dz = dv.get<float>(B);
-    float* lv = dv.get<float>(B);
+    float* scr = dv.get<float>(GradScratch::floats(B));
     float* la = dv.get<float>(epochs);
-    if (!dx || !dy || !dw || !dg || !m || !v || !idx || !H1 || !H2 || !dH1 || !dH2 || !dz || !lv || !la)
-        return AMR_ERR_CUDA;
+    if (!dx || !dy || !dw || !m || !v || !idx || !scr || !la) return AMR_ERR_CUDA;
+    const GradScratch sc(scr, B);
     cudaMemcpyAsync(dx, X, n * K * sizeof(float), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(dy, y, n * sizeof(float), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(dw, weights, nw * sizeof(float), cudaMemcpyHostToDevice, s);
@@ -396,12 +631,10 @@ int amr_mlp_train(int dim, const float* X, const float* y, long n, float pw, int
         const long b = (long)((z >> 32) % (uint64_t)n);
         k_perm<<<blocks(n), 256, 0, s>>>(idx, n, a % n, b);
         for (long bi = 0; bi < nb; ++bi) {
-            if (fwd_bwd(dim, dx, idx + bi * B, dy, B, pw, dw, dg, la + ep, 1.0f / (float)(B * nb), H1, H2, dz, lv,
-                        dH1, dH2, s))
-                return AMR_ERR_CUDA;
             ++step;
-            const float c1 = 1.f - powf(0.9f, (float)step), c2 = 1.f - powf(0.999f, (float)step);
-            k_adam<<<blocks(nw), 256, 0, s>>>(dw, dg, m, v, nw, lr, c1, c2);
+            const AdamStep adam{dw, m, v, lr, 1.f - powf(0.9f, (float)step), 1.f - powf(0.999f, (float)step)};
+            if (fwd_bwd(dim, dx, idx + bi * B, dy, B, pw, dw, nullptr, la + ep, 1.0f / (float)(B * nb), 1, sc, adam, s))
+                return AMR_ERR_CUDA;
         }
     }
     if (cudaGetLastError() != cudaSuccess) return AMR_ERR_CUDA;
@@ -420,14 +653,14 @@ int amr_mlp_train(int dim, const float* X, const float* y, long n, float pw, int
 // buffers the runtime maps for it, and an allocation behind the runtime's back
 // can fail or fragment its pool), code issuing work while a CUDA stream
 // capture is in progress (allocation is not allowed there), and real-time
-// loops where an allocation may synchronise the device. For them the hidden
-// activations of the forward/backward pass live in the fixed array below,
-// which every GPU that loads this library holds until the process exits:
-// 4 x 2048 x 64 + 2 x 2048 + 64 floats (about 2.1 MB).
+// loops where an allocation may synchronise the device. For them the scratch
+// of the forward/backward pass lives in the fixed array below, which every GPU
+// that loads this library holds until the process exits: GradScratch of 2048
+// rows (2048 x 64 + 32 x 4290 + 160000 floats, about 1.7 MB).
 // ---------------------------------------------------------------------------
 namespace {
 constexpr long NOALLOC_ROWS = AMR_MLP_NOALLOC_MAX_ROWS;
-constexpr size_t NOALLOC_FLOATS = 4 * NOALLOC_ROWS * MLP_H + 2 * NOALLOC_ROWS + 64;
+constexpr size_t NOALLOC_FLOATS = GradScratch::floats(NOALLOC_ROWS);
 }  // namespace
 
 static __device__ __align__(256) float g_noalloc_scratch[NOALLOC_FLOATS];
@@ -458,20 +691,7 @@ extern "C" int amr_mlp_grad_noalloc(int dim, const float* X, const float* y, lon
     if (cudaGetDevice(&dev) != cudaSuccess) return AMR_ERR_CUDA;
     float* base = noalloc_scratch(dev);
     if (!base) return AMR_ERR_CUDA;
-    const size_t hs = (size_t)NOALLOC_ROWS * MLP_H;
-    float* H1 = base;
-    float* H2 = base + hs;
-    float* dH1 = base + 2 * hs;
-    float* dH2 = base + 3 * hs;
-    float* dz = base + 4 * hs;
-    float* lv = dz + NOALLOC_ROWS;
-    float* lacc = lv + NOALLOC_ROWS;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // the loss accumulator keeps the previous call's value: clear it
-    if (cudaMemsetAsync(lacc, 0, sizeof(float), s) != cudaSuccess) return AMR_ERR_CUDA;
-    if (fwd_bwd(dim, X, nullptr, y, (int)n, pos_weight, weights, grad, lacc, 1.0f / (float)n, H1, H2, dz, lv, dH1,
-                dH2, s))
-        return AMR_ERR_CUDA;
-    if (cudaMemcpyAsync(loss, lacc, sizeof(float), cudaMemcpyDeviceToDevice, s) != cudaSuccess) return AMR_ERR_CUDA;
-    return cudaGetLastError() == cudaSuccess ? AMR_OK : AMR_ERR_CUDA;
+    return fwd_bwd(dim, X, nullptr, y, n, pos_weight, weights, grad, loss, 1.0f / (float)n, 0, GradScratch(base, n),
+                   AdamStep{}, s);
 }
