@@ -18,12 +18,15 @@ namespace amr {
 // arithmetic helpers: FP64 uses IEEE division and square root; FP32 uses the
 // fast approximate forms (the FP32 path is compared by tolerance, not bits)
 // ---------------------------------------------------------------------------
+// half(a, b): a / 2 + b with a / 2 exact, so the fused form rounds as the two operations do
 template <typename T> struct Num;
 template <> struct Num<double> {
+    __device__ __forceinline__ static double half(double a, double b) { return __fma_rn(0.5, a, b); }
     __device__ __forceinline__ static double div(double a, double b) { return a / b; }
     __device__ __forceinline__ static double sqr(double a) { return sqrt(a); }
 };
 template <> struct Num<float> {
+    __device__ __forceinline__ static float half(float a, float b) { return 0.5f * a + b; }
     __device__ __forceinline__ static float div(float a, float b) { return __fdividef(a, b); }
     __device__ __forceinline__ static float sqr(float a) { return sqrtf(a); }
 };
@@ -68,6 +71,12 @@ template <> struct Vec16<double> {
         *reinterpret_cast<double2*>(p) = make_double2(o[0], o[1]);
     }
 };
+
+// a normal power of two, whose reciprocal is exact
+__device__ __forceinline__ bool exact_reciprocal(double x) {
+    return (__double_as_longlong(x) & 0xFFFFFFFFFFFFFll) == 0;
+}
+__device__ __forceinline__ bool exact_reciprocal(float) { return true; }
 
 // slot coordinate of local index l in an active (d < D) or inactive dimension
 template <int D>
@@ -118,34 +127,53 @@ __device__ __forceinline__ double pressure_d(const double* U, double gm1) {
 // (Sec. 3.2): quadratic candidates, linear weights (1, 10, 5)/16, Jiang-Shu
 // smoothness indicators, alpha_k = d_k / (eps + beta_k)^2, eps = 1e-6
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ T weno5(T a, T b, T c, T d, T e) {
-    const T q0 = (T(3) * a - T(10) * b + T(15) * c) * T(0.125);
-    const T q1 = (-b + T(6) * c + T(3) * d) * T(0.125);
-    const T q2 = (T(3) * c + T(6) * d - e) * T(0.125);
-    const T t0 = a - T(2) * b + c;
-    const T s0 = a - T(4) * b + T(3) * c;
-    const T t1 = b - T(2) * c + d;
-    const T s1 = b - d;
-    const T t2 = c - T(2) * d + e;
-    const T s2 = T(3) * c - T(4) * d + e;
-    const T c1312 = T(13.0 / 12.0);
-    const T b0 = c1312 * (t0 * t0) + T(0.25) * (s0 * s0);
-    const T b1 = c1312 * (t1 * t1) + T(0.25) * (s1 * s1);
-    const T b2 = c1312 * (t2 * t2) + T(0.25) * (s2 * s2);
-    const T e0 = T(1.0e-6) + b0;
-    const T e1 = T(1.0e-6) + b1;
-    const T e2 = T(1.0e-6) + b2;
-    const T a0 = Num<T>::div(T(0.0625), e0 * e0);
-    const T a1 = Num<T>::div(T(0.625), e1 * e1);
-    const T a2 = Num<T>::div(T(0.3125), e2 * e2);
-    return Num<T>::div(a0 * q0 + a1 * q1 + a2 * q2, a0 + a1 + a2);
+// FP64: left- (nodes 0..4) and right-biased (nodes 5..1) values of one face. The
+// FP64 pipe issues one warp instruction per SM every 9.2 ns (1/64 of the FP32
+// rate), whatever else the kernel does, so the count of FP64 instructions is
+// the time, and a division costs 7.6 of them. Bit for bit the formulas
+//   q0 = (3a - 10b + 15c) / 8, q1 = (-b + 6c + 3d) / 8, q2 = (3c + 6d - e) / 8,
+//   t0 = a - 2b + c, t1 = b - 2c + d, t2 = c - 2d + e,
+//   s0 = a - 4b + 3c, s1 = b - d, s2 = 3c - 4d + e,
+//   beta_k = 13/12 t_k^2 + s_k^2 / 4, alpha_k = d_k / (eps + beta_k)^2,
+//   (alpha_0 q0 + alpha_1 q1 + alpha_2 q2) / (alpha_0 + alpha_1 + alpha_2),
+// evaluated left to right with one rounding per operation: a factor that is a
+// power of two is exact, so it goes into a fused multiply-add without changing
+// a rounding (6c is twice the rounded 3c, -2b, -4b and s^2 / 4 are exact) or
+// out of the sums (the 1/8 of the candidates and the 1/16 of the linear
+// weights, applied to the quotient), and the rounded 3c, 3d are shared between
+// candidates, indicators and the two sides. 74 instruction slots per value
+// instead of 92; k_rhs in FP64: 3D 4.60 -> 3.96 ms at 120 leaves of 16^3, 2D
+// 1.12 -> 0.99 ms at 808 leaves of 16^2.
+__device__ __forceinline__ double weno5_side(double a, double b, double c, double d, double e, double c3, double d3) {
+    const double q0 = (3.0 * a - 10.0 * b) + 15.0 * c;
+    const double q1 = __fma_rn(2.0, c3, -b) + d3;
+    const double q2 = __fma_rn(2.0, d3, c3) - e;
+    const double t0 = __fma_rn(-2.0, b, a) + c;
+    const double t1 = __fma_rn(-2.0, c, b) + d;
+    const double t2 = __fma_rn(-2.0, d, c) + e;
+    const double s0 = __fma_rn(-4.0, b, a) + c3;
+    const double s1 = b - d;
+    const double s2 = __fma_rn(-4.0, d, c3) + e;
+    const double c1312 = 13.0 / 12.0;
+    const double e0 = 1.0e-6 + __fma_rn(0.25, s0 * s0, c1312 * (t0 * t0));
+    const double e1 = 1.0e-6 + __fma_rn(0.25, s1 * s1, c1312 * (t1 * t1));
+    const double e2 = 1.0e-6 + __fma_rn(0.25, s2 * s2, c1312 * (t2 * t2));
+    const double a0 = __drcp_rn(e0 * e0);                  // 16 alpha_k
+    const double a1 = 10.0 / (e1 * e1);
+    const double a2 = 5.0 / (e2 * e2);
+    return (a0 * q0 + a1 * q1 + a2 * q2) / (a0 + a1 + a2) * 0.125;
+}
+__device__ __forceinline__ void weno5_pair(double v0, double v1, double v2, double v3, double v4, double v5,
+                                           double& left, double& right) {
+    const double m2 = 3.0 * v2, m3 = 3.0 * v3;
+    left = weno5_side(v0, v1, v2, v3, v4, m2, m3);
+    right = weno5_side(v5, v4, v3, v2, v1, m3, m2);
 }
 
 // FP32: left- (nodes 0..4) and right-biased (nodes 5..1) WENO5-JS values of one
 // face together; the right stencil is the left one mirrored, so two candidate
 // values and two smoothness terms are shared between them. Same formulas as
-// weno5. FAST: the normalised weights are unchanged when every alpha_k is
+// in FP64. FAST: the normalised weights are unchanged when every alpha_k is
 // multiplied by e0^2 e1^2 e2^2, which leaves a single division, exact up to
 // rounding while no product overflows: checked on the division's operands, a
 // finite numerator and a denominator below 2^126, the range of the fast
@@ -293,8 +321,7 @@ __device__ __forceinline__ void weno5_lr(const T (&w)[6], T& left, T& right, boo
     if constexpr (sizeof(T) == 4) {
         weno5_pair<FAST>(w[0], w[1], w[2], w[3], w[4], w[5], left, right, ok);
     } else {
-        left = weno5(w[0], w[1], w[2], w[3], w[4]);
-        right = weno5(w[5], w[4], w[3], w[2], w[1]);
+        weno5_pair(w[0], w[1], w[2], w[3], w[4], w[5], left, right);
     }
 }
 
@@ -378,7 +405,7 @@ __device__ __forceinline__ void face_flux(const T (&p)[6], const T (&un)[6], con
             const T v = side ? utR[j] : utL[j];
             usq = usq + v * v;
         }
-        const T E = Num<T>::div(ps, gm1) + T(0.5) * rho * usq;
+        const T E = Num<T>::half(rho * usq, Num<T>::div(ps, gm1));
         const T mn = rho * uns;
         T* Uo = side ? UR : UL;
         T* Fo = side ? FR : FL;
@@ -431,7 +458,7 @@ __device__ __forceinline__ void face_flux(const T (&p)[6], const T (&un)[6], con
     }
     const T hS = T(0.5) * fmax(sR, sL);
 #pragma unroll
-    for (int v = 0; v < NF; ++v) F[v] = T(0.5) * (FR[v] + FL[v]) - hS * (UR[v] - UL[v]);
+    for (int v = 0; v < NF; ++v) F[v] = Num<T>::half(FR[v] + FL[v], -(hS * (UR[v] - UL[v])));
 }
 
 // ---------------------------------------------------------------------------
@@ -1045,18 +1072,20 @@ __device__ __forceinline__ T restrict_mean(const T (&ch)[1 << D]) {
 // central scheme, whose divergence reads the faces at i -+ 3/2)
 // PADQ: per-variable blocks and the halo block start on 128-byte boundaries
 // (the halo planes are then tensor-copy destinations)
-template <int D, int N, int DZ, int EXT = 0, bool PADQ = false> struct Chunk {
+// DY: rows per chunk (2D/3D)
+template <int D, int N, int DZ, int DY, int EXT = 0, bool PADQ = false> struct Chunk {
     static constexpr int S = N + 2 * G;
-    static constexpr int CX = N, CY = D >= 2 ? N : 1, CZ = D == 3 ? DZ : 1;
-    // staged cells per variable: 1D/2D the whole slot; 3D the DZ centre planes
-    // in full (S x S) and the 2G halo planes only over the interior N x N, the
-    // only part the z-faces read
-    static constexpr int QX = S, QY = D >= 2 ? S : 1, QZ = D == 3 ? DZ : 1;
+    static constexpr int CX = N, CY = D >= 2 ? DY : 1, CZ = D == 3 ? DZ : 1;
+    // staged cells per variable: 1D/2D the chunk's rows with their ghosts; 3D
+    // the DZ centre planes (DY + 2G rows of S cells) and the 2G halo planes
+    // only over the chunk's N x DY columns, the only part the z-faces read
+    static constexpr int QX = S, QY = D >= 2 ? DY + 2 * G : 1, QZ = D == 3 ? DZ : 1;
     static constexpr int QC = PADQ ? (QX * QY * QZ + 31) / 32 * 32 : QX * QY * QZ;   // centre cells
-    static constexpr int QH = D == 3 ? 2 * G * N * N : 0;         // compact halo cells
+    static constexpr int QH = D == 3 ? 2 * G * N * DY : 0;        // compact halo cells
     static constexpr int QN = PADQ ? (QC + QH + 31) / 32 * 32 : QC + QH;
     static constexpr int CELLS = CX * CY * CZ;
-    static constexpr int NCH = D == 3 ? N / DZ : 1;
+    static constexpr int NCHY = D >= 2 ? N / DY : 1;              // chunks of a patch along y, in all
+    static constexpr int NCH = (D == 3 ? N / DZ : 1) * NCHY;
     static constexpr int F0 = (CX + 1 + EXT) * CY * CZ;
     static constexpr int F1 = D >= 2 ? CX * (CY + 1 + EXT) * CZ : 0;
     static constexpr int F2 = D == 3 ? CX * CY * (CZ + 1 + EXT) : 0;
@@ -1071,9 +1100,9 @@ template <int D, int N, int DZ, int EXT = 0, bool PADQ = false> struct Chunk {
     static constexpr int TRANS = D == 1 ? 1 : (D == 2 ? N : N * N);   // cells on a patch face
 };
 
-template <typename T, int D, int N, int DZ, int FLUX, bool TMA = false>
+template <typename T, int D, int N, int DZ, int DY, int FLUX, bool TMA = false>
 constexpr size_t rhs_smem_bytes() {
-    using C = Chunk<D, N, DZ, FLUX == AMR_FLUX_CENTRAL ? 2 : 0, TMA>;
+    using C = Chunk<D, N, DZ, DY, FLUX == AMR_FLUX_CENTRAL ? 2 : 0, TMA>;
     // TMA: 128 bytes to align the base, an mbarrier and an abort word
     return sizeof(T) * ((size_t)(D + 2) * C::QN + (size_t)(D + 2) * C::FMAX) + (TMA ? 128 + 16 : 0);
 }
@@ -1119,15 +1148,16 @@ __device__ __forceinline__ bool rhs_mbar_wait(uint32_t mbar, uint32_t parity, vo
 // the same-level neighbour across z or the slot itself), issued by thread 0
 // while the other threads stage the centre planes; they land as conserved
 // variables in the halo block and are converted to primitives in place.
-template <typename T, int D, int N, int DZ, int NTH, int MINB, int FLUX, bool TMA = false>
+template <typename T, int D, int N, int DZ, int DY, int NTH, int MINB, int FLUX, bool TMA = false>
 __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__ Us, const T* U0,
                                              T* Uout, T* __restrict__ faces,
                                              int stage, int one_slot, int fuse_restrict,
                                              const __grid_constant__ CUtensorMap tmap) {
     constexpr bool CEN = FLUX == AMR_FLUX_CENTRAL;
     constexpr int EXT = CEN ? 2 : 0;                   // central: faces i - 3/2 .. N + 1/2 along d
-    static_assert(!TMA || (D == 3 && DZ >= 4 && sizeof(T) == 4 && !CEN), "halo boxes with one source slot");
-    using C = Chunk<D, N, DZ, EXT, TMA>;
+    static_assert(!TMA || (D == 3 && DZ >= 4 && DY == N && sizeof(T) == 4 && !CEN), "halo boxes with one source slot");
+    static_assert(D < 2 || (N % DY == 0 && DY % 2 == 0), "chunks of whole coarse rows");
+    using C = Chunk<D, N, DZ, DY, EXT, TMA>;
     constexpr int NV = D + 2;
     constexpr int NT = D - 1;
     constexpr int CPT = (C::CELLS + NTH - 1) / NTH;
@@ -1161,7 +1191,9 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
     const int n_items = npatch * C::NCH;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int pi = item / C::NCH;
-        const int z0 = (item - pi * C::NCH) * DZ;        // first interior plane of the chunk (3D)
+        const int ch0 = item - pi * C::NCH;
+        const int z0 = ch0 / C::NCHY * DZ;               // first interior plane (3D) and row of the chunk
+        const int y0 = D >= 2 ? ch0 % C::NCHY * DY : 0;
         const int slot = one_slot >= 0 ? one_slot : g.leaf_list[pi];
         const int lev = g.level[slot];
         const int pf = g.pflag[slot];
@@ -1247,14 +1279,14 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                 const int sz = D == 3 ? z0 + G + qz : 0;
                 const int x0 = (xv + XV0) * VE - XP;
                 T Uv[NV][VE];
-                const int ly = qy - G;
+                const int ly = y0 + qy - G, sy = y0 + qy;
                 if (D >= 2 && (ly < 0 || ly >= N)) {
-                    loadv(Uv, ly < 0 ? sym : syp, sz, qy + (ly < 0 ? dym : dyp), x0);
+                    loadv(Uv, ly < 0 ? sym : syp, sz, sy + (ly < 0 ? dym : dyp), x0);
                 } else {
-                    loadv(Uv, slot, sz, qy, x0);
+                    loadv(Uv, slot, sz, sy, x0);
                     if (x0 < G) {                            // x ghosts below the interior
                         T Wv[NV][VE];
-                        loadv(Wv, sxm, sz, qy, x0 + dxm);
+                        loadv(Wv, sxm, sz, sy, x0 + dxm);
 #pragma unroll
                         for (int e = 0; e < VE; ++e)
                             if (x0 + e < G) {
@@ -1264,7 +1296,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                     }
                     if (x0 + VE > G + N) {                   // x ghosts above the interior
                         T Wv[NV][VE];
-                        loadv(Wv, sxp, sz, qy, x0 + dxp);
+                        loadv(Wv, sxp, sz, sy, x0 + dxp);
 #pragma unroll
                         for (int e = 0; e < VE; ++e)
                             if (x0 + e >= G + N) {
@@ -1311,18 +1343,18 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                 across(2, 0, szm, dzm);
                 across(2, 1, szp, dzp);
 #pragma unroll 2
-                for (int iv = threadIdx.x; iv < NHV * N * 2 * G; iv += NTH) {
-                    const int xv = iv % NHV, hy = (iv / NHV) % N, zh = iv / (NHV * N);
+                for (int iv = threadIdx.x; iv < NHV * DY * 2 * G; iv += NTH) {
+                    const int xv = iv % NHV, hy = (iv / NHV) % DY, zh = iv / (NHV * DY);
                     const int sz = z0 + (zh < G ? zh : zh + DZ);
                     const int lz = sz - G;
                     const int src = lz < 0 ? szm : (lz >= N ? szp : slot);
                     const int shz = lz < 0 ? dzm : (lz >= N ? dzp : 0);
                     T Uv[NV][VE];
-                    loadv(Uv, src, sz + shz, hy + G, HX0 + xv * VE);
+                    loadv(Uv, src, sz + shz, y0 + hy + G, HX0 + xv * VE);
 #pragma unroll
                     for (int e = 0; e < VE; ++e) {
                         const int x = HX0 + xv * VE + e;
-                        if (x >= G && x < G + N) stage(Uv, e, C::QC + (zh * N + hy) * N + (x - G));
+                        if (x >= G && x < G + N) stage(Uv, e, C::QC + (zh * DY + hy) * N + (x - G));
                     }
                 }
             }
@@ -1335,7 +1367,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
             constexpr int ROWS = NV * C::CZ * C::CY;
             for (int r = threadIdx.x; r < ROWS; r += NTH) {
                 const int v = r / (C::CZ * C::CY), rz = (r / C::CY) % C::CZ, ry = r % C::CY;
-                const T* a = U0 + slot_index(g, slot, v, D == 3 ? z0 + G + rz : 0, D >= 2 ? ry + G : 0, G);
+                const T* a = U0 + slot_index(g, slot, v, D == 3 ? z0 + G + rz : 0, D >= 2 ? y0 + ry + G : 0, G);
                 asm volatile("prefetch.global.L2 [%0];\n" ::"l"(a));
             }
         }
@@ -1393,7 +1425,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                             const int zz = fk + k - EXT / 2;     // staged z index 0 .. DZ + 5
                             id = (zz >= G && zz < G + DZ)
                                      ? ((zz - G) * C::QY + fj + G) * C::QX + fi + G
-                                     : C::QC + ((zz < G ? zz : zz - DZ) * N + fj) * N + fi;
+                                     : C::QC + ((zz < G ? zz : zz - DZ) * DY + fj) * N + fi;
                         }
                         pp[k] = q[id];
                         un[k] = q[(1 + DD) * C::QN + id];
@@ -1432,13 +1464,13 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                     for (int v = 0; v < NV; ++v) Fs[v * C::FMAX + fp] = Fg[v];
                     // patch-boundary faces needed by the coarse-fine flux correction
                     // (central: the conservative face values, saved by the divergence)
-                    const int fd = DD == 0 ? fi : (DD == 1 ? fj : fk + z0);
+                    const int fd = DD == 0 ? fi : (DD == 1 ? fj + y0 : fk + z0);
                     const int side = fd == 0 ? 0 : (fd == N ? 1 : -1);
                     if (!CEN && side >= 0 && ((pf >> (8 + 2 * DD + side)) & 1)) {
                         int tidx;
                         if constexpr (D == 1) tidx = 0;
-                        else if constexpr (D == 2) tidx = DD == 0 ? fj : fi;
-                        else tidx = DD == 0 ? (fk + z0) * N + fj : (DD == 1 ? (fk + z0) * N + fi : fj * N + fi);
+                        else if constexpr (D == 2) tidx = DD == 0 ? fj + y0 : fi;
+                        else tidx = DD == 0 ? (fk + z0) * N + fj + y0 : (DD == 1 ? (fk + z0) * N + fi : (fj + y0) * N + fi);
                         T* dst = faces + ((long long)slot * 2 * D + 2 * DD + side) * NV * C::TRANS + tidx;
 #pragma unroll
                         for (int v = 0; v < NV; ++v) dst[v * C::TRANS] = Fg[v];
@@ -1465,6 +1497,9 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                 const T* Fd = Fs + (d == 1 ? C::F0 : 0);
                 const T dxd = T(g.dx[lev][d]);
                 const T idx = T(1) / dxd;                        // FP32: multiply by the reciprocal
+                // FP64: the same where the reciprocal of dx is exact (dx a power
+                // of two), as the product then rounds as the quotient does
+                const bool by_idx = sizeof(T) == 4 || exact_reciprocal(dxd);
                 constexpr int fstep = d == 0 ? 1 : (d == 1 ? FX : FX * FY);
 #pragma unroll
                 for (int n = 0; n < CPT; ++n) {
@@ -1477,15 +1512,15 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                         const int fhi = flo + fstep;
                         if constexpr (CEN) {
                             // Eq. 9 as the difference of G = (26 F_f - F_{f-1} - F_{f+1}) / 24
-                            const int cd = d == 0 ? ci : (d == 1 ? cj : ck + z0);
+                            const int cd = d == 0 ? ci : (d == 1 ? cj + y0 : ck + z0);
                             const int side = cd == 0 ? 0 : (cd == N - 1 ? 1 : -1);
                             const bool save = side >= 0 && ((pf >> (8 + 2 * d + side)) & 1);
                             T* dst = nullptr;
                             if (save) {
                                 int tidx;
                                 if (D == 1) tidx = 0;
-                                else if (D == 2) tidx = d == 0 ? cj : ci;
-                                else tidx = d == 0 ? (ck + z0) * N + cj : (d == 1 ? (ck + z0) * N + ci : cj * N + ci);
+                                else if (D == 2) tidx = d == 0 ? cj + y0 : ci;
+                                else tidx = d == 0 ? (ck + z0) * N + cj + y0 : (d == 1 ? (ck + z0) * N + ci : (cj + y0) * N + ci);
                                 dst = faces + ((long long)slot * 2 * D + 2 * d + side) * NV * C::TRANS + tidx;
                             }
 #pragma unroll
@@ -1498,14 +1533,14 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                                 else { glo = glo / T(24); ghi = ghi / T(24); }
                                 if (save) dst[v * C::TRANS] = side ? ghi : glo;
                                 const T df = ghi - glo;
-                                const T dv = sizeof(T) == 4 ? df * idx : df / dxd;
+                                const T dv = by_idx ? df * idx : df / dxd;
                                 R[n][v] = d == 0 ? -dv : R[n][v] - dv;
                             }
                         } else {
 #pragma unroll
                             for (int v = 0; v < NV; ++v) {
                                 const T df = Fd[v * C::FMAX + fhi] - Fd[v * C::FMAX + flo];
-                                const T dv = sizeof(T) == 4 ? df * idx : df / dxd;
+                                const T dv = by_idx ? df * idx : df / dxd;
                                 R[n][v] = d == 0 ? -dv : R[n][v] - dv;
                             }
                         }
@@ -1535,7 +1570,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                 const int ci = cidx % C::CX;
                 const int cj = (cidx / C::CX) % C::CY;
                 const int ck = cidx / (C::CX * C::CY);
-                const int sx = ci + G, sy = D >= 2 ? cj + G : 0, sz = D == 3 ? z0 + ck + G : 0;
+                const int sx = ci + G, sy = D >= 2 ? y0 + cj + G : 0, sz = D == 3 ? z0 + ck + G : 0;
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
                     const long long id = slot_index(g, slot, v, sz, sy, sx);
@@ -1551,7 +1586,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
         // 4. fused restriction of the chunk's cells into the parent
         if (fuse) {
             constexpr int H = N / 2;
-            constexpr int HZ = D == 3 ? DZ / 2 : 1, HY = D >= 2 ? H : 1;
+            constexpr int HZ = D == 3 ? DZ / 2 : 1, HY = D >= 2 ? DY / 2 : 1;
             constexpr int NCC = HZ * HY * H;                // coarse cells of the chunk
             static_assert(D < 3 || DZ % 2 == 0, "chunks hold whole coarse planes");
             __syncthreads();
@@ -1560,7 +1595,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
                 if (threadIdx.x == 0) atomicOr(&g.time->err, ERR_MESH);
             } else {
                 const int ox = (g.coord[slot * 3 + 0] & 1) * H;
-                const int oy = D >= 2 ? (g.coord[slot * 3 + 1] & 1) * H : 0;
+                const int oy = D >= 2 ? (g.coord[slot * 3 + 1] & 1) * H + y0 / 2 : 0;
                 const int oz = D == 3 ? (g.coord[slot * 3 + 2] & 1) * H + z0 / 2 : 0;
                 for (int c = threadIdx.x; c < NV * NCC; c += NTH) {
                     const int v = c / NCC, r = c - v * NCC;
@@ -1590,7 +1625,7 @@ template <typename T, int D, int N>
 __global__ void __launch_bounds__(256) k_reflux(Grid g, T* Uout, const T* __restrict__ faces, int stage,
                                                 int one_item) {
     constexpr int NV = D + 2;
-    constexpr int TRANS = Chunk<D, N, 1>::TRANS;
+    constexpr int TRANS = Chunk<D, N, 1, N>::TRANS;
     if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
     const T rb = stage == 0 ? T(1) : (stage == 1 ? T(0.25) : T(2.0 / 3.0));
     const T dt = T(g.time->dt);

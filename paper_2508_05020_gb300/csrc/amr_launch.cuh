@@ -13,6 +13,7 @@ template <typename T, int D, int N, int V = 0> struct RhsCfg {
     // buffer), two CTAs of at most 128 registers per SM; otherwise two-plane
     // chunks
     static constexpr int DZ = D == 3 ? (sizeof(T) == 4 && N == 16 ? 4 : 2) : 1;
+    static constexpr int DY = N;
     static constexpr int NTH = D == 1 ? 64 : 256;
     static constexpr int MINB = (D == 3 && sizeof(T) == 4) ? (N == 16 ? 2 : 3) : 1;
     static constexpr bool TMA = false;
@@ -24,19 +25,19 @@ template <typename T, int D, int N, int V = 0> struct RhsCfg {
 // with the halo planes brought in by tensor copies (TMA) while the threads
 // stage the centre planes
 template <> struct RhsCfg<float, 3, 16, 1> {
-    static constexpr int DZ = 2, NTH = 256, MINB = 3;
+    static constexpr int DZ = 2, DY = 16, NTH = 256, MINB = 3;
     static constexpr bool TMA = false;
 };
 template <> struct RhsCfg<float, 3, 16, 2> {
-    static constexpr int DZ = 8, NTH = 512, MINB = 1;
+    static constexpr int DZ = 8, DY = 16, NTH = 512, MINB = 1;
     static constexpr bool TMA = false;
 };
 template <> struct RhsCfg<float, 3, 16, 3> {
-    static constexpr int DZ = 4, NTH = 256, MINB = 2;
+    static constexpr int DZ = 4, DY = 16, NTH = 256, MINB = 2;
     static constexpr bool TMA = true;
 };
 template <> struct RhsCfg<float, 3, 16, 4> {
-    static constexpr int DZ = 8, NTH = 512, MINB = 1;
+    static constexpr int DZ = 8, DY = 16, NTH = 512, MINB = 1;
     static constexpr bool TMA = true;
 };
 template <typename T, int D, int N, int FLUX> struct RhsShapes {
@@ -64,8 +65,8 @@ static cudaError_t rhs_launch_v(const Grid& g, const T* Us, const T* U0, T* Uout
     using C = RhsCfg<T, D, N, V>;
     static const CUtensorMap none{};                     // the kernels without tensor copies ignore it
     if (C::TMA && !tmap) return cudaErrorInvalidValue;   // no tensor map of this state array
-    k_rhs<T, D, N, C::DZ, C::NTH, C::MINB, FLUX, C::TMA>
-        <<<grid, C::NTH, rhs_smem_bytes<T, D, N, C::DZ, FLUX, C::TMA>(), s>>>(g, Us, U0, Uout, faces, stage,
+    k_rhs<T, D, N, C::DZ, C::DY, C::NTH, C::MINB, FLUX, C::TMA>
+        <<<grid, C::NTH, rhs_smem_bytes<T, D, N, C::DZ, C::DY, FLUX, C::TMA>(), s>>>(g, Us, U0, Uout, faces, stage,
                                                                           one_slot, fuse, tmap ? *tmap : none);
     return cudaSuccess;
 }
@@ -104,9 +105,9 @@ static cudaError_t rhs_launch(const Grid& g, const T* Us, const T* U0, T* Uout, 
 template <typename T, int D, int N, int FLUX, int V>
 static cudaError_t rhs_prepare_v() {
     using C = RhsCfg<T, D, N, V>;
-    return cudaFuncSetAttribute(k_rhs<T, D, N, C::DZ, C::NTH, C::MINB, FLUX, C::TMA>,
+    return cudaFuncSetAttribute(k_rhs<T, D, N, C::DZ, C::DY, C::NTH, C::MINB, FLUX, C::TMA>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)rhs_smem_bytes<T, D, N, C::DZ, FLUX, C::TMA>());
+                                (int)rhs_smem_bytes<T, D, N, C::DZ, C::DY, FLUX, C::TMA>());
 }
 
 template <typename T, int D, int N, int FLUX>
