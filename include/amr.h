@@ -146,7 +146,9 @@ typedef struct {
 /* Launch parameters of the batched step (amr_get_tuning), in this order:
  * CTAs per SM of the ghost fill, ghost cells per ghost-fill work item, CTAs per
  * SM of the fused RHS, the reflux, the restriction, the CFL reduction and the
- * plain flagging. */
+ * plain flagging. Until amr_autotune or amr_set_tuning chooses another RHS
+ * grid or tile shape than the default (2, 0), the RHS's grid follows a rule of
+ * the library by precision, dimension and patch size. */
 #define AMR_TUNE_GHOST_GRID 0
 #define AMR_TUNE_GHOST_CHUNK 1
 #define AMR_TUNE_RHS_GRID 2

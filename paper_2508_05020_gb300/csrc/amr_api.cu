@@ -44,6 +44,9 @@ struct amr_ctx {
     // item), the defaults or the autotuner's choice (AMR_TUNE_* order)
     int tune[AMR_TUNE_N] = {16, 128, 2, 4, 8, 8, 4, 0};
     float tune_ms[AMR_TUNE_N] = {0, 0, 0, 0, 0, 0, 0, 0};
+    // the RHS's grid and tile shape were chosen (autotuner, amr_set_tuning);
+    // before that its grid follows the kernel's own rule (Kernels::rhs_grid)
+    bool rhs_tuned = false;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     // hierarchy
@@ -87,9 +90,10 @@ struct amr_ctx {
     int n_ghost = 0, n_ghost_face = 0;
     Grid grid{};
     // graph
-    // captured step graphs by [CFL step][stage-1 ghost fill skipped]
-    cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-    long long graph_kernels[2][2] = {{0, 0}, {0, 0}};
+    // captured step graphs by [class of the RHS launch][CFL step][stage-1 ghost fill skipped]
+    // (a graph serves any hierarchy; the class is the launch that suits it)
+    cudaGraphExec_t graph[RHS_CLASSES][2][2] = {};
+    long long graph_kernels[RHS_CLASSES][2][2] = {};
     // the ghosts of U0 hold the values the first stage's ghost fill would
     // write (a regrid filled them at the current time and left the mesh as it was)
     bool ghosts_valid = false;
@@ -375,15 +379,24 @@ void assign_slots(amr_ctx* c, const std::vector<Key>& created, const std::vector
 
 int grid_size(const amr_ctx* c, int per_sm) { return c->nsm * per_sm; }
 
+// class and grid of the fused RHS for the present hierarchy
+template <typename T>
+RhsPlan rhs_plan(const amr_ctx* c) {
+    RhsPlan p = Kernels<T>::rhs_plan(c->grid, c->n_leaf, c->nsm);
+    if (c->rhs_tuned) p.grid = grid_size(c, c->tune[AMR_TUNE_RHS_GRID]);
+    return p;
+}
+
 // request-list entries read back with the counts (longer lists take a second read-back)
 constexpr int REQ_READ = 2048;
 
 void drop_graphs(amr_ctx* c) {
-    for (auto& row : c->graph)
-        for (auto& ex : row) {
-            if (ex) cudaGraphExecDestroy(ex);
-            ex = nullptr;
-        }
+    for (auto& cls : c->graph)
+        for (auto& row : cls)
+            for (auto& ex : row) {
+                if (ex) cudaGraphExecDestroy(ex);
+                ex = nullptr;
+            }
 }
 
 template <typename T>
@@ -457,6 +470,7 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
         k += 2;
     }
     const double tfrac[3] = {0.0, 1.0, 0.5};
+    const RhsPlan plan = rhs_plan<T>(c);
     for (int s = 0; s < 3; ++s) {
         T* src = St<T>(c, s == 0 ? 0 : s);
         T* dst = St<T>(c, s == 0 ? 1 : (s == 1 ? 2 : 0));
@@ -468,9 +482,8 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
             ++k;
         }
         CK(mark(c->ev[s][1]), "event");
-        CK(Kernels<T>::rhs_stage(g, src, St<T>(c, 0), dst, reinterpret_cast<T*>(c->faces), s,
-                                 grid_size(c, c->tune[AMR_TUNE_RHS_GRID]),
-                                 c->stream, -1, 1, tmap_of(c, src)),
+        CK(Kernels<T>::rhs_stage(g, src, St<T>(c, 0), dst, reinterpret_cast<T*>(c->faces), s, plan.grid, c->stream, -1, 1,
+                                 tmap_of(c, src), plan.cls),
            "rhs stage");
         CK(mark(c->ev[s][2]), "event");
         CK(Kernels<T>::reflux(g, dst, reinterpret_cast<T*>(c->faces), s, grid_size(c, c->tune[AMR_TUNE_REFLUX_GRID]),
@@ -572,8 +585,9 @@ int step_impl(amr_ctx* c, double dt, double* dt_used) {
         if (r) return r;
     } else if (c->use_graph) {
         const bool skip = c->ghosts_valid;
-        cudaGraphExec_t& ex = c->graph[with_cfl][skip];
-        long long& nk = c->graph_kernels[with_cfl][skip];
+        const int cls = rhs_plan<T>(c).cls;
+        cudaGraphExec_t& ex = c->graph[cls][with_cfl][skip];
+        long long& nk = c->graph_kernels[cls][with_cfl][skip];
         if (!ex) {
             cudaGraph_t gr;
             CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
@@ -1005,7 +1019,7 @@ int autotune_impl(amr_ctx* c) {
     if (err == cudaSuccess) {                            // fused RHS: tile shape x grid, timed on a stage
         // that reads only its input (A -> B) and one that also reads U0 and
         // writes in place (B, U0 = A -> A, as the step's last stage does)
-        const int shapes = Kernels<T>::rhs_shapes(g);
+        const int shapes = Kernels<T>::rhs_shapes(g), cls = rhs_plan<T>(c).cls;
         float bestv = 1e30f;
         int best_shape = 0, best_grid = c->tune[AMR_TUNE_RHS_GRID];
         for (int sh = 0; sh < shapes && err == cudaSuccess; ++sh) {
@@ -1021,10 +1035,10 @@ int autotune_impl(amr_ctx* c) {
                     nk += 2;
                     const cudaError_t e =
                         Kernels<T>::rhs_stage(g, A, St<T>(c, 0), B, faces, 0, grid_size(c, gr), c->stream, -1, 1,
-                                              tmap_of(c, A));
+                                              tmap_of(c, A), cls);
                     if (e != cudaSuccess) return e;
                     return Kernels<T>::rhs_stage(g, B, A, A, faces, 2, grid_size(c, gr), c->stream, -1, 1,
-                                                 tmap_of(c, B));
+                                                 tmap_of(c, B), cls);
                 }, t);
                 if (t < bestv) {
                     bestv = t;
@@ -1035,6 +1049,7 @@ int autotune_impl(amr_ctx* c) {
         }
         c->tune[AMR_TUNE_RHS_SHAPE] = best_shape;
         c->tune[AMR_TUNE_RHS_GRID] = best_grid;
+        c->rhs_tuned = true;
         c->grid.rhs_shape = best_shape;
         c->tune_ms[AMR_TUNE_RHS_SHAPE] = c->tune_ms[AMR_TUNE_RHS_GRID] = bestv;
     }
@@ -1664,6 +1679,9 @@ int amr_set_tuning(amr_ctx* c, const int params[AMR_TUNE_N]) {
         else ok = v >= 1 && v <= 64;
         if (!ok) return fail(c, AMR_ERR_ARG, "launch parameter out of range");
     }
+    // the values an untuned context reports, set again, leave the RHS untuned
+    c->rhs_tuned = c->rhs_tuned || params[AMR_TUNE_RHS_GRID] != c->tune[AMR_TUNE_RHS_GRID] ||
+                   params[AMR_TUNE_RHS_SHAPE] != c->tune[AMR_TUNE_RHS_SHAPE];
     for (int i = 0; i < AMR_TUNE_N; ++i) c->tune[i] = params[i];
     c->grid.rhs_shape = c->tune[AMR_TUNE_RHS_SHAPE];
     drop_graphs(c);

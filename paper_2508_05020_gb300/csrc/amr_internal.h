@@ -94,6 +94,16 @@ struct Grid {
     DevTime* time;
 };
 
+// How many leaf patches a launch of the fused RHS has, which decides its chunks
+// and its grid (any choice computes the same): RHS_FEW leave most SMs without
+// a chunk, RHS_PAIR are at most two chunks per SM, RHS_SOME make a few waves,
+// RHS_MANY more
+enum { RHS_FEW = 0, RHS_PAIR = 1, RHS_SOME = 2, RHS_MANY = 3, RHS_CLASSES = 4 };
+struct RhsPlan {
+    int cls;                    // RHS_*
+    int grid;                   // CTAs of an untuned launch
+};
+
 // Kernel set of one storage precision. Implemented for float and double in
 // amr_f32.cu / amr_f64.cu; the FP64 unit is compiled without FMA contraction.
 template <typename T>
@@ -111,6 +121,8 @@ struct Kernels {
                                   cudaStream_t s, int one_slot, int chunk = 512, bool stage_only = false);
     // compiled tile-shape candidates of the fused RHS for this grid and flux
     static int rhs_shapes(const Grid& g);
+    // how a hierarchy of `leaves` leaf patches (in a pool of g.cap) is advanced with tile shape 0
+    static RhsPlan rhs_plan(const Grid& g, int leaves, int nsm);
     // RHS + SSP-RK3 stage of every patch (or one patch if one_slot >= 0);
     // fuse_restrict: patches of the finest level L - 1 also restrict their
     // output into their parents (the restriction of level L - 1 is then done)
@@ -118,7 +130,7 @@ struct Kernels {
     // tile shapes that copy halo planes with TMA (else cudaErrorInvalidValue)
     static cudaError_t rhs_stage(const Grid& g, const T* Us, const T* U0, T* Uout, T* faces,
                                  int stage, int grid, cudaStream_t s, int one_slot, int fuse_restrict = 0,
-                                 const void* tmap = nullptr);
+                                 const void* tmap = nullptr, int cls = RHS_MANY);
     static cudaError_t reflux(const Grid& g, T* Uout, const T* faces, int stage, int grid,
                               cudaStream_t s, int one_slot);
     // covered cells of level-1 patches from the children of level `level`
