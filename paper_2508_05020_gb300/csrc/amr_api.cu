@@ -6,10 +6,12 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <new>
 #include <set>
 #include <string>
@@ -90,10 +92,14 @@ struct amr_ctx {
     int n_ghost = 0, n_ghost_face = 0;
     Grid grid{};
     // graph
-    // captured step graphs by [class of the RHS launch][CFL step][stage-1 ghost fill skipped]
-    // (a graph serves any hierarchy; the class is the launch that suits it)
-    cudaGraphExec_t graph[RHS_CLASSES][2][2] = {};
-    long long graph_kernels[RHS_CLASSES][2][2] = {};
+    // captured step graphs by (size class, CFL step, stage-1 ghost fill skipped):
+    // a graph serves any hierarchy, the class (the bit length of the patch count
+    // and the class of the RHS launch) decides the grids that suit it
+    struct StepGraph {
+        cudaGraphExec_t exec = nullptr;
+        long long kernels = 0;
+    };
+    std::map<std::array<int, 4>, StepGraph> graphs;
     // the ghosts of U0 hold the values the first stage's ghost fill would
     // write (a regrid filled them at the current time and left the mesh as it was)
     bool ghosts_valid = false;
@@ -379,6 +385,35 @@ void assign_slots(amr_ctx* c, const std::vector<Key>& created, const std::vector
 
 int grid_size(const amr_ctx* c, int per_sm) { return c->nsm * per_sm; }
 
+// Bit length of the patch count: a step's grids are sized for up to
+// 2^(bits) - 1 patches, so that small hierarchies launch no idle CTAs (2432
+// empty CTAs of a ghost fill cost 2 us), and change only when the count leaves
+// its power of two
+int size_bits(const amr_ctx* c) {
+    int b = 0;
+    while (((long long)c->canon.size() >> b) > 0) ++b;
+    return b;
+}
+// CTAs of 256 threads for `per_patch` threads per patch, at most per_sm CTAs per SM
+int grid_for(const amr_ctx* c, int per_sm, long long per_patch) {
+    const long long most = std::min<long long>(1ll << size_bits(c), c->cap);
+    return (int)std::max<long long>(1, std::min<long long>(grid_size(c, per_sm), (most * per_patch + 255) / 256));
+}
+// threads per patch of the ghost fills (a warp per work item), the CFL
+// reduction (16-byte vectors of cells) and the restriction (coarse cells)
+long long ghost_threads(const amr_ctx* c, bool stage_only) {
+    const int chunk = c->tune[AMR_TUNE_GHOST_CHUNK];
+    const int face = c->n_ghost_face / (2 * c->dim);
+    return 32ll * (stage_only ? 2 * c->dim * ((face + chunk - 1) / chunk) : (c->n_ghost + chunk - 1) / chunk);
+}
+long long patch_cells(const amr_ctx* c) {
+    long long n = 1;
+    for (int d = 0; d < c->dim; ++d) n *= c->N;
+    return n;
+}
+long long cfl_threads(const amr_ctx* c) { return patch_cells(c) * (c->precision / 8) / 16; }
+long long restrict_threads(const amr_ctx* c) { return patch_cells(c) >> c->dim; }
+
 // class and grid of the fused RHS for the present hierarchy
 template <typename T>
 RhsPlan rhs_plan(const amr_ctx* c) {
@@ -391,12 +426,9 @@ RhsPlan rhs_plan(const amr_ctx* c) {
 constexpr int REQ_READ = 2048;
 
 void drop_graphs(amr_ctx* c) {
-    for (auto& cls : c->graph)
-        for (auto& row : cls)
-            for (auto& ex : row) {
-                if (ex) cudaGraphExecDestroy(ex);
-                ex = nullptr;
-            }
+    for (auto& gr : c->graphs)
+        if (gr.second.exec) cudaGraphExecDestroy(gr.second.exec);
+    c->graphs.clear();
 }
 
 template <typename T>
@@ -443,16 +475,22 @@ bool encode_tmaps(amr_ctx* c) {
 
 template <typename T>
 int fill_all_levels(amr_ctx* c, T* U, double tfrac) {
-    for (int l = 0; l < c->L; ++l) {
-        CK(Kernels<T>::ghost_fill(c->grid, U, l, tfrac, grid_size(c, c->tune[AMR_TUNE_GHOST_GRID]), c->stream, -1,
-                                  c->tune[AMR_TUNE_GHOST_CHUNK]),
-           "ghost fill");
-        ++c->kernels;
-    }
+    CK(Kernels<T>::ghost_fill(c->grid, U, tfrac,
+                              grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, false)), c->stream, -1,
+                              c->tune[AMR_TUNE_GHOST_CHUNK]),
+       "ghost fill");
+    ++c->kernels;
     return AMR_OK;
 }
 
 // Enqueue one SSP-RK3 step of the batched mode (optionally with the CFL step).
+// A small hierarchy's step is its launches (about 3 us each), so there are few:
+// one ghost fill for all levels (it reads interior cells only), dt set by the
+// CFL reduction's last block, the time moved on by the last RHS, no reflux with
+// one level: 13 launches with three levels where one per level and scalar made
+// 21 (1D FP32, four levels: 92 -> 51 us per step). Programmatic dependences between
+// them gained 1 to 3 %, and cost FP64 runs up to 40 %, as the early CTAs of an
+// RHS pile up on few SMs.
 template <typename T>
 int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
     const Grid& g = c->grid;
@@ -464,42 +502,42 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
     };
     if (with_cfl) {
         CK(mark(c->ev_cfl[0]), "event");
-        CK(Kernels<T>::cfl(g, St<T>(c, 0), grid_size(c, c->tune[AMR_TUNE_CFL_GRID]), c->stream, -1), "cfl");
-        CK(launch_finalize_dt(g, c->stream), "finalize dt");
+        CK(Kernels<T>::cfl(g, St<T>(c, 0), grid_for(c, c->tune[AMR_TUNE_CFL_GRID], cfl_threads(c)), c->stream, -1, true),
+           "cfl");
         CK(mark(c->ev_cfl[1]), "event");
-        k += 2;
+        ++k;
     }
     const double tfrac[3] = {0.0, 1.0, 0.5};
     const RhsPlan plan = rhs_plan<T>(c);
+    const int gghost = grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, true));
+    const int greflux = grid_for(c, c->tune[AMR_TUNE_REFLUX_GRID], 256);
+    const int grestrict = grid_for(c, c->tune[AMR_TUNE_RESTRICT_GRID], restrict_threads(c));
     for (int s = 0; s < 3; ++s) {
         T* src = St<T>(c, s == 0 ? 0 : s);
         T* dst = St<T>(c, s == 0 ? 1 : (s == 1 ? 2 : 0));
         CK(mark(c->ev[s][0]), "event");
-        for (int l = 0; l < c->L && !(s == 0 && skip_fill0); ++l) {
-            CK(Kernels<T>::ghost_fill(g, src, l, tfrac[s], grid_size(c, c->tune[AMR_TUNE_GHOST_GRID]), c->stream, -1,
-                                      c->tune[AMR_TUNE_GHOST_CHUNK], true),
+        if (!(s == 0 && skip_fill0)) {
+            CK(Kernels<T>::ghost_fill(g, src, tfrac[s], gghost, c->stream, -1, c->tune[AMR_TUNE_GHOST_CHUNK], true),
                "ghost fill");
             ++k;
         }
         CK(mark(c->ev[s][1]), "event");
-        CK(Kernels<T>::rhs_stage(g, src, St<T>(c, 0), dst, reinterpret_cast<T*>(c->faces), s, plan.grid, c->stream, -1, 1,
-                                 tmap_of(c, src), plan.cls),
+        CK(Kernels<T>::rhs_stage(g, src, St<T>(c, 0), dst, reinterpret_cast<T*>(c->faces), s, plan.grid, c->stream, -1,
+                                 RHS_RESTRICT | (s == 2 ? RHS_ADVANCE : 0), tmap_of(c, src), plan.cls),
            "rhs stage");
         CK(mark(c->ev[s][2]), "event");
-        CK(Kernels<T>::reflux(g, dst, reinterpret_cast<T*>(c->faces), s, grid_size(c, c->tune[AMR_TUNE_REFLUX_GRID]),
-                              c->stream, -1),
-           "reflux");
+        ++k;
+        if (c->L > 1) {
+            CK(Kernels<T>::reflux(g, dst, reinterpret_cast<T*>(c->faces), s, greflux, c->stream, -1), "reflux");
+            ++k;
+        }
         CK(mark(c->ev[s][3]), "event");
-        k += 2;
         for (int l = c->L - 2; l >= 1; --l) {             // level L - 1: fused into the RHS
-            CK(Kernels<T>::restrict_level(g, dst, l, grid_size(c, c->tune[AMR_TUNE_RESTRICT_GRID]), c->stream, -1),
-               "restrict");
+            CK(Kernels<T>::restrict_level(g, dst, l, grestrict, c->stream, -1), "restrict");
             ++k;
         }
         CK(mark(c->ev[s][4]), "event");
     }
-    CK(launch_advance_time(g.time, c->stream), "advance time");
-    ++k;
     if (nk) *nk = k;
     return AMR_OK;
 }
@@ -520,12 +558,10 @@ int per_patch_step(amr_ctx* c, bool with_cfl) {
     for (int s = 0; s < 3; ++s) {
         T* src = St<T>(c, s == 0 ? 0 : s);
         T* dst = St<T>(c, s == 0 ? 1 : (s == 1 ? 2 : 0));
-        for (int l = 0; l < c->L; ++l)
-            for (int i = c->level_off_h[l]; i < c->level_off_h[l + 1]; ++i) {
-                CK(Kernels<T>::ghost_fill(g, src, l, tfrac[s], 8, c->stream, c->canon_slot[i], 512, true),
-                   "ghost fill");
-                ++c->kernels;
-            }
+        for (int slot : c->canon_slot) {
+            CK(Kernels<T>::ghost_fill(g, src, tfrac[s], 8, c->stream, slot, 512, true), "ghost fill");
+            ++c->kernels;
+        }
         for (size_t i = 0; i < c->canon_slot.size(); ++i) {
             CK(Kernels<T>::rhs_stage(g, src, St<T>(c, 0), dst, reinterpret_cast<T*>(c->faces), s, 8, c->stream,
                                      c->canon_slot[i], 0, tmap_of(c, src)),
@@ -585,9 +621,9 @@ int step_impl(amr_ctx* c, double dt, double* dt_used) {
         if (r) return r;
     } else if (c->use_graph) {
         const bool skip = c->ghosts_valid;
-        const int cls = rhs_plan<T>(c).cls;
-        cudaGraphExec_t& ex = c->graph[cls][with_cfl][skip];
-        long long& nk = c->graph_kernels[cls][with_cfl][skip];
+        amr_ctx::StepGraph& sg = c->graphs[{size_bits(c), rhs_plan<T>(c).cls, with_cfl, skip}];
+        cudaGraphExec_t& ex = sg.exec;
+        long long& nk = sg.kernels;
         if (!ex) {
             cudaGraph_t gr;
             CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
@@ -921,6 +957,7 @@ int set_state_impl(amr_ctx* c, int n, const int* levels, const int* coords, cons
     c->time_h->lam = 0ull;
     c->time_h->err = 0;
     c->time_h->cancel = 0;
+    c->time_h->ticket = 0u;
     CK(cudaMemcpyAsync(c->time_d, c->time_h, sizeof(DevTime), cudaMemcpyHostToDevice, c->stream), "set time");
     CK(cudaStreamSynchronize(c->stream), "set time");
     return AMR_OK;
@@ -999,13 +1036,8 @@ int autotune_impl(amr_ctx* c) {
             for (int ch : chunks) {
                 float t = 0.f;
                 err = timed([&]() {
-                    for (int l = 0; l < c->L; ++l) {
-                        const cudaError_t e = Kernels<T>::ghost_fill(g, A, l, 0.0, grid_size(c, gr), c->stream, -1, ch,
-                                                                     true);
-                        ++nk;
-                        if (e != cudaSuccess) return e;
-                    }
-                    return cudaSuccess;
+                    ++nk;
+                    return Kernels<T>::ghost_fill(g, A, 0.0, grid_size(c, gr), c->stream, -1, ch, true);
                 }, t);
                 if (err != cudaSuccess) break;
                 if (t < bestv) {
@@ -1075,7 +1107,7 @@ int autotune_impl(amr_ctx* c) {
         const int cands[] = {2, 4, 8, 16, 32};
         err = tune_one(AMR_TUNE_CFL_GRID, cands, 5, [&](int gr) {
             ++nk;
-            return Kernels<T>::cfl(g, A, grid_size(c, gr), c->stream, -1);
+            return Kernels<T>::cfl(g, A, grid_size(c, gr), c->stream, -1, false);
         });
     }
     if (err == cudaSuccess) {                            // plain flagging of A (scratch flags)
@@ -1746,7 +1778,7 @@ int amr_get_timing(amr_ctx* c, double ms[AMR_TIMING_SLOTS], int launches[AMR_TIM
     if (launches) {
         const int rt = c->regrid_timed ? 1 : 0;
         // restriction: levels L-2..1 per stage (level L-1 is restricted inside the RHS launch)
-        const int l[AMR_TIMING_SLOTS] = {3 * c->L, 3, 3, 3 * std::max(c->L - 2, 0), c->cfl_timed ? 2 : 0, rt, 0, 0,
+        const int l[AMR_TIMING_SLOTS] = {3, 3, c->L > 1 ? 3 : 0, 3 * std::max(c->L - 2, 0), c->cfl_timed ? 1 : 0, rt, 0, 0,
                                          rt * c->regrid_fill_launches, 0};
         for (int i = 0; i < AMR_TIMING_SLOTS; ++i) launches[i] = l[i];
     }

@@ -5,20 +5,8 @@
 
 namespace amr {
 
-// dt = CFL / lambda_max (Sec. 3.1: the sound speed sets the step), clipped to
-// t_end; the maximum is reset for the next step.
 __global__ void k_finalize_dt(DevTime* tm, double cfl, double t_end) {
-    if (tm->cancel) return;
-    const double lam = __longlong_as_double((long long)tm->lam);
-    if (!(lam > 0.0) || !(lam <= 1.0e300)) {
-        tm->err |= ERR_NONFINITE;
-        tm->dt = 0.0;
-    } else {
-        double dt = cfl / lam;
-        if (t_end > 0.0) dt = fmin(dt, t_end - tm->t);
-        tm->dt = dt;
-    }
-    tm->lam = 0ull;
+    if (!tm->cancel) finalize_dt(tm, tm->lam, cfl, t_end);
 }
 
 __global__ void k_set_dt(DevTime* tm, double dt) {

@@ -26,6 +26,10 @@ constexpr int ERR_NONFINITE = 1;
 constexpr int ERR_MESH = 2;
 constexpr int ERR_TIMEOUT = 4;        // a bounded device wait gave up
 
+// flags of a launch of the fused RHS: patches of the finest level also restrict
+// their output into their parents; the time moves on by dt (a step's last stage)
+constexpr int RHS_RESTRICT = 1, RHS_ADVANCE = 2;
+
 // limit of a bounded wait of the tensor-core pipeline, in SM clock cycles
 // (about two seconds)
 constexpr long long TC_WAIT_CYCLES = 1ll << 32;
@@ -39,7 +43,25 @@ struct DevTime {
     int cancel;                 // nonzero: the kernels of a step return at once (set by the request
                                 // compaction when the mesh may change; a step issued ahead of that
                                 // decision is then void and issued again)
+    unsigned ticket;            // blocks of the CFL reduction that are done (its last block resets it)
 };
+
+#ifdef __CUDACC__
+// dt = CFL / lambda_max (Sec. 3.1: the sound speed sets the step), clipped to
+// t_end; the maximum is reset for the next step
+__device__ __forceinline__ void finalize_dt(DevTime* tm, unsigned long long lam_bits, double cfl, double t_end) {
+    const double lam = __longlong_as_double((long long)lam_bits);
+    if (!(lam > 0.0) || !(lam <= 1.0e300)) {
+        atomicOr(&tm->err, ERR_NONFINITE);
+        tm->dt = 0.0;
+    } else {
+        double dt = cfl / lam;
+        if (t_end > 0.0) dt = fmin(dt, t_end - tm->t);
+        tm->dt = dt;
+    }
+    tm->lam = 0ull;
+}
+#endif
 
 // Read-only description of the grid and the metadata tables, passed by value.
 struct Grid {
@@ -111,32 +133,32 @@ struct Kernels {
     // one-time kernel attributes (dynamic shared memory); call before any capture
     static cudaError_t prepare(const Grid& g);
     static cudaError_t prepare_mlp(const Grid& g);
-    // ghost cells of every patch of `level` (same-level copy, prolongation,
-    // physical boundaries) at time t + tfrac * dt
+    // ghost cells of every patch (same-level copy, prolongation, physical
+    // boundaries) at time t + tfrac * dt
     // stage_only: the face ghosts without a same-level neighbour across their
     // face (all a stage reads from a slot's ghost region: the RHS and the
     // prolongation read same-level neighbours' interiors directly); else every
     // ghost cell (what the flag stencils read)
-    static cudaError_t ghost_fill(const Grid& g, T* U, int level, double tfrac, int grid,
+    static cudaError_t ghost_fill(const Grid& g, T* U, double tfrac, int grid,
                                   cudaStream_t s, int one_slot, int chunk = 512, bool stage_only = false);
     // compiled tile-shape candidates of the fused RHS for this grid and flux
     static int rhs_shapes(const Grid& g);
     // how a hierarchy of `leaves` leaf patches (in a pool of g.cap) is advanced with tile shape 0
     static RhsPlan rhs_plan(const Grid& g, int leaves, int nsm);
     // RHS + SSP-RK3 stage of every patch (or one patch if one_slot >= 0);
-    // fuse_restrict: patches of the finest level L - 1 also restrict their
-    // output into their parents (the restriction of level L - 1 is then done)
+    // flags: RHS_RESTRICT (the restriction of level L - 1 is then done), RHS_ADVANCE
     // tmap: the tensor map (CUtensorMap) of the state array Us, needed by the
     // tile shapes that copy halo planes with TMA (else cudaErrorInvalidValue)
     static cudaError_t rhs_stage(const Grid& g, const T* Us, const T* U0, T* Uout, T* faces,
-                                 int stage, int grid, cudaStream_t s, int one_slot, int fuse_restrict = 0,
+                                 int stage, int grid, cudaStream_t s, int one_slot, int flags = 0,
                                  const void* tmap = nullptr, int cls = RHS_MANY);
     static cudaError_t reflux(const Grid& g, T* Uout, const T* faces, int stage, int grid,
                               cudaStream_t s, int one_slot);
     // covered cells of level-1 patches from the children of level `level`
     static cudaError_t restrict_level(const Grid& g, T* U, int level, int grid, cudaStream_t s,
                                       int one_slot);
-    static cudaError_t cfl(const Grid& g, const T* U, int grid, cudaStream_t s, int one_slot);
+    // finalize: the step too, as launch_finalize_dt sets it
+    static cudaError_t cfl(const Grid& g, const T* U, int grid, cudaStream_t s, int one_slot, bool finalize = false);
     static cudaError_t init_ic(const Grid& g, T* U, const int* list, int n, cudaStream_t s);
     static cudaError_t prolong_new(const Grid& g, T* U, const int* list, int n, cudaStream_t s);
     static cudaError_t flag_plain(const Grid& g, const T* U, int* anyflag, int grid,

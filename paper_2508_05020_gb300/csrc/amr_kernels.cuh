@@ -690,9 +690,12 @@ __device__ __forceinline__ void load_meta_warp(const Grid& g, int slot, PatchMet
 // child has rho <= 0 or p <= 0.
 // ---------------------------------------------------------------------------
 // NBR_READS (the ghost fill): C +- e_d outside Q is read from Q's same-level
-// neighbour when it exists, as a stage leaves that face ghost of Q unfilled;
-// otherwise (new patches in a regrid, which may create that neighbour in the
-// same launch) from Q's ghost cells, filled before the mesh changed.
+// neighbour, which R2 provides inside the domain (Q and every in-domain
+// neighbour of Q that a slope reaches lie in the Moore neighbourhood of the
+// parent, which has children); outside the domain it is the boundary rule's
+// value. So the fill reads interior cells only and all levels go in one
+// launch. Otherwise (new patches in a regrid, which may create that neighbour
+// in the same launch) from Q's ghost cells, filled before the mesh changed.
 // The coarse cell C of fine local cell l: returns Q, the patch that holds C
 // (from the parent's neighbour table; -1 if there is none), and sets C's
 // local coordinates Lc in Q and the child index s of l (bit d: the upper half
@@ -718,10 +721,51 @@ __device__ __forceinline__ int prolong_locate(const PatchMeta& m, const int* l, 
     return m.par >= 0 ? m.pnbr[(oc[2] + 1) * 9 + (oc[1] + 1) * 3 + (oc[0] + 1)] : -1;
 }
 
-// U_C and the minmod slopes of coarse cell Lc of Q (NBR_READS: see below)
+// time and double-Mach states of a fill's boundary rules
+struct BcState {
+    double t;
+    const double *pre, *post;                            // (rho, u, v, p)
+};
+
+// The boundary rule of kind `kind` at a ghost cell whose global x index is Gx
+// (level lev): true if it sets a fixed state (conserved, in out); otherwise it
+// copies (outflow) or mirrors
+template <typename T, int D>
+__device__ __forceinline__ bool bc_fixed(const Grid& g, int kind, int lev, int Gx, const BcState& b, T* out) {
+    bool dirichlet = false, behind = false;
+    if (kind == AMR_BC_DMR_INFLOW) {
+        dirichlet = true;
+        behind = true;
+    } else if (kind == AMR_BC_DMR_BOTTOM || kind == AMR_BC_DMR_TOP) {
+        const double x = g.lo[0] + ((double)Gx + 0.5) * g.dx[lev][0];
+        if (kind == AMR_BC_DMR_BOTTOM) {
+            behind = x < 1.0 / 6.0;
+            dirichlet = behind;
+        } else {
+            behind = x < 1.0 / 6.0 + (1.0 + 20.0 * b.t) / sqrt(3.0);
+            dirichlet = true;
+        }
+    }
+    if (dirichlet) {
+        const double* st = behind ? b.post : b.pre;
+        const double r = st[0], ux = st[1], uy = st[2], pp = st[3];
+        const double usq = ux * ux + uy * uy;
+        double Uc[4];
+        Uc[0] = r;
+        Uc[1] = r * ux;
+        Uc[2] = r * uy;
+        Uc[3] = pp / (g.gamma - 1.0) + 0.5 * r * usq;
+#pragma unroll
+        for (int v = 0; v < D + 2; ++v) out[v] = T(v < 4 ? Uc[v] : 0.0);
+    }
+    return dirichlet;
+}
+
+// U_C and the minmod slopes of coarse cell Lc of Q (NBR_READS: see above; the
+// double-Mach rules exist in 2D only)
 template <typename T, int D, int N, bool NBR_READS>
-__device__ __forceinline__ void prolong_slopes(const Grid& g, const T* U, int Q, const int* Lc, T (&UC)[D + 2],
-                                               T (&slope)[D][D + 2]) {
+__device__ __forceinline__ void prolong_slopes(const Grid& g, const T* U, int Q, const int* Lc, const BcState& bc,
+                                               T (&UC)[D + 2], T (&slope)[D][D + 2]) {
     constexpr int NV = D + 2;
     const int bx = sc<D>(0, Lc[0]), by = sc<D>(1, Lc[1]), bz = sc<D>(2, Lc[2]);
 #pragma unroll
@@ -732,18 +776,40 @@ __device__ __forceinline__ void prolong_slopes(const Grid& g, const T* U, int Q,
         // C +- e_d outside Q: see NBR_READS
         long long ip = slot_index(g, Q, 0, bz + ez, by + ey, bx + ex);
         long long im = slot_index(g, Q, 0, bz - ez, by - ey, bx - ex);
+        bool outp = false, outm = false;
         if (NBR_READS && Lc[d] == N - 1) {
             const int qn = g.nbr[Q * NBR + 13 + (d == 0 ? 1 : (d == 1 ? 3 : 9))];
             if (qn >= 0) ip = slot_index(g, qn, 0, bz - (N - 1) * ez, by - (N - 1) * ey, bx - (N - 1) * ex);
+            else outp = true;
+            if (qn == -1) atomicOr(&g.time->err, ERR_MESH);
         }
         if (NBR_READS && Lc[d] == 0) {
             const int qn = g.nbr[Q * NBR + 13 - (d == 0 ? 1 : (d == 1 ? 3 : 9))];
             if (qn >= 0) im = slot_index(g, qn, 0, bz + (N - 1) * ez, by + (N - 1) * ey, bx + (N - 1) * ex);
+            else outm = true;
+            if (qn == -1) atomicOr(&g.time->err, ERR_MESH);
+        }
+        // outside the domain: C's own value (outflow), that with the normal
+        // momentum turned (mirror), or a fixed state
+        T fixed[D == 2 ? NV : 1];
+        bool mirror = false, isfixed = false;
+        if (NBR_READS && (outp || outm)) {
+            const int kind = g.bc[d][outp ? 1 : 0];
+            if constexpr (D == 2) isfixed = bc_fixed<T, D>(g, kind, g.level[Q], g.coord[Q * 3] * N + Lc[0], bc, fixed);
+            mirror = !isfixed && kind != AMR_BC_OUTFLOW;
         }
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-            const T up = U[ip + (long long)v * g.slot_elems];
-            const T um = U[im + (long long)v * g.slot_elems];
+            T up, um;
+            if (NBR_READS && (outp || outm)) {
+                const T c = v == 1 + d && mirror ? -UC[v] : UC[v];
+                const T o = D == 2 && isfixed ? fixed[D == 2 ? v : 0] : c;
+                up = outp ? o : U[ip + (long long)v * g.slot_elems];
+                um = outm ? o : U[im + (long long)v * g.slot_elems];
+            } else {
+                up = U[ip + (long long)v * g.slot_elems];
+                um = U[im + (long long)v * g.slot_elems];
+            }
             const T a = up - UC[v];
             const T b = UC[v] - um;
             const T pick = fabs(a) <= fabs(b) ? a : b;
@@ -783,7 +849,7 @@ __device__ __forceinline__ bool prolong_positive(const Grid& g, const T (&UC)[D 
 }
 
 template <typename T, int D, int N, bool NBR_READS>
-__device__ void prolong_cell(const Grid& g, const T* U, const PatchMeta& m, const int* l, T* out) {
+__device__ void prolong_cell(const Grid& g, const T* U, const PatchMeta& m, const int* l, const BcState& bc, T* out) {
     constexpr int NV = D + 2;
     int Lc[3], s[3];
     const int Q = prolong_locate<D, N>(m, l, Lc, s);
@@ -794,7 +860,7 @@ __device__ void prolong_cell(const Grid& g, const T* U, const PatchMeta& m, cons
         return;
     }
     T UC[NV], slope[D][NV];
-    prolong_slopes<T, D, N, NBR_READS>(g, U, Q, Lc, UC, slope);
+    prolong_slopes<T, D, N, NBR_READS>(g, U, Q, Lc, bc, UC, slope);
     const bool ok = prolong_positive<T, D>(g, UC, slope);
     int mine = 0;
 #pragma unroll
@@ -807,7 +873,7 @@ __device__ void prolong_cell(const Grid& g, const T* U, const PatchMeta& m, cons
 
 // value of an in-domain cell of a patch: interior, same-level neighbour or prolongation
 template <typename T, int D, int N>
-__device__ void in_domain_value(const Grid& g, const T* U, const PatchMeta& m, const int* l, T* out) {
+__device__ void in_domain_value(const Grid& g, const T* U, const PatchMeta& m, const int* l, const BcState& bc, T* out) {
     constexpr int NV = D + 2;
     const int slot = m.slot;
     int o[3] = {0, 0, 0};
@@ -830,7 +896,7 @@ __device__ void in_domain_value(const Grid& g, const T* U, const PatchMeta& m, c
         for (int v = 0; v < NV; ++v) out[v] = U[slot_index(g, nb, v, sz, sy, sx)];
         return;
     }
-    prolong_cell<T, D, N, true>(g, U, m, l, out);
+    prolong_cell<T, D, N, true>(g, U, m, l, bc, out);
 }
 
 // Ghost value of local cell l of a patch: physical boundary rules applied from
@@ -838,9 +904,7 @@ __device__ void in_domain_value(const Grid& g, const T* U, const PatchMeta& m, c
 // boundary dimension by dimension in the order x, y, z), then the in-domain
 // value of the mapped cell.
 template <typename T, int D, int N>
-__device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* l, double t, T* out,
-                            const double* pre, const double* post) {
-    constexpr int NV = D + 2;
+__device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* l, const BcState& bc, T* out) {
     const int lev = m.lev;
     const int* c = m.c;
     int neg = 0;
@@ -858,31 +922,7 @@ __device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* 
         const int kind = g.bc[dd][side];
         const int Gd = c[dd] * N + l[dd];
         const int n = g.ext[lev][dd] * N;
-        bool dirichlet = false, behind = false;
-        if (kind == AMR_BC_DMR_INFLOW) {
-            dirichlet = true;
-            behind = true;
-        } else if (kind == AMR_BC_DMR_BOTTOM || kind == AMR_BC_DMR_TOP) {
-            const double x = g.lo[0] + ((double)(c[0] * N + l[0]) + 0.5) * g.dx[lev][0];
-            if (kind == AMR_BC_DMR_BOTTOM) {
-                behind = x < 1.0 / 6.0;
-                dirichlet = behind;
-            } else {
-                behind = x < 1.0 / 6.0 + (1.0 + 20.0 * t) / sqrt(3.0);
-                dirichlet = true;
-            }
-        }
-        if (dirichlet) {
-            const double* st = behind ? post : pre;     // (rho, u, v, p)
-            const double r = st[0], ux = st[1], uy = st[2], pp = st[3];
-            const double usq = ux * ux + uy * uy;
-            double Uc[4];
-            Uc[0] = r;
-            Uc[1] = r * ux;
-            Uc[2] = r * uy;
-            Uc[3] = pp / (g.gamma - 1.0) + 0.5 * r * usq;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) out[v] = T(v < 4 ? Uc[v] : 0.0);
+        if (bc_fixed<T, D>(g, kind, lev, c[0] * N + l[0], bc, out)) {
 #pragma unroll
             for (int d = 0; d < D; ++d)
                 if ((neg >> d) & 1) out[1 + d] = -out[1 + d];
@@ -897,14 +937,14 @@ __device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* 
         }
         l[dd] = Gs - c[dd] * N;
     }
-    in_domain_value<T, D, N>(g, U, m, l, out);
+    in_domain_value<T, D, N>(g, U, m, l, bc, out);
 #pragma unroll
     for (int d = 0; d < D; ++d)
         if ((neg >> d) & 1) out[1 + d] = -out[1 + d];
 }
 
 // ---------------------------------------------------------------------------
-// K1-K3: ghost fill of every patch of one level. The regrid fills every ghost
+// K1-K3: ghost fill of every patch of every level. The regrid fills every ghost
 // cell (the slot-order table); a stage (stage_only) fills the face boxes that
 // have no same-level neighbour across them (coarse-fine and domain sides),
 // whose cells the RHS reads from the slot (the box-order table that follows
@@ -914,7 +954,7 @@ __device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* 
 // shared-memory copy; warps never wait for one another.
 // ---------------------------------------------------------------------------
 template <typename T, int D, int N, bool STAGE>
-__global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(Grid g, T* U, int level, double tfrac, int one_slot,
+__global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(Grid g, T* U, double tfrac, int one_slot,
                                                double4 pre, double4 post, int chunk, int n_cells) {
     constexpr bool stage_only = STAGE;                  // compiled apart: the full fill keeps its registers
     constexpr int NV = D + 2;
@@ -922,11 +962,10 @@ __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(
     if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     PatchMeta& m = metas[warp];
-    const int lo = g.level_off[level], hi = g.level_off[level + 1];
-    const int npatch = one_slot >= 0 ? 1 : hi - lo;
-    const double t = g.time->t + tfrac * g.time->dt;
+    const int npatch = one_slot >= 0 ? 1 : g.counts[0];
     const double pr[4] = {pre.x, pre.y, pre.z, pre.w};
     const double po[4] = {post.x, post.y, post.z, post.w};
+    const BcState bc{g.time->t + tfrac * g.time->dt, pr, po};
     // a stage walks the 2d face boxes of a patch (G N^(d-1) table entries
     // each) and skips a box whole when a same-level neighbour lies across it
     constexpr int BOX = G * (D == 1 ? 1 : (D == 2 ? N : N * N));
@@ -941,7 +980,7 @@ __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(
         const int run = rest / nchunk;
         const int g0 = run * span + (rest - run * nchunk) * chunk;
         const int g1 = min(g0 + chunk, run * span + span);
-        const int slot = one_slot >= 0 ? one_slot : g.all_list[lo + pi];
+        const int slot = one_slot >= 0 ? one_slot : g.all_list[pi];
         if (stage_only) {
             const int d = run >> 1, side = run & 1;
             const int across = g.nbr[slot * NBR + 13 + (side ? 1 : -1) * (d == 0 ? 1 : (d == 1 ? 3 : 9))];
@@ -976,7 +1015,7 @@ __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(
                     if (Q < 0) {
                         atomicOr(&g.time->err, ERR_MESH);
                     } else {
-                        prolong_slopes<T, D, N, true>(g, U, Q, Lc, UC, slope);
+                        prolong_slopes<T, D, N, true>(g, U, Q, Lc, bc, UC, slope);
                         ok = prolong_positive<T, D>(g, UC, slope);
                     }
 #pragma unroll
@@ -1015,7 +1054,7 @@ __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(
             int l[3] = {(pk & 1023) - G, ((pk >> 10) & 1023) - G, ((pk >> 20) & 1023) - G};
             const int sx = l[0] + G, sy = D >= 2 ? l[1] + G : 0, sz = D == 3 ? l[2] + G : 0;
             T val[NV];
-            ghost_value<T, D, N>(g, U, m, l, t, val, pr, po);
+            ghost_value<T, D, N>(g, U, m, l, bc, val);
 #pragma unroll
             for (int v = 0; v < NV; ++v) U[slot_index(g, slot, v, sz, sy, sx)] = val[v];
         }
@@ -1062,7 +1101,7 @@ __device__ __forceinline__ T restrict_mean(const T (&ch)[1 << D]) {
 // dimension at a time go to a shared buffer; each thread accumulates the
 // divergence of its own cells in registers, then writes
 // U_out = a U0 + b (U_s + dt R)  (a = 0, b = 1 in stage 1).
-// fuse_restrict: a chunk of a patch of the finest level L - 1 (>= 1) also
+// RHS_RESTRICT in flags: a chunk of a patch of the finest level L - 1 (>= 1) also
 // restricts its updated cells into the parent (restrict_mean, as the
 // restriction kernel does): the finest level is never the coarse side of a
 // reflux, so its stage output is final here, and its parent, whose cells are
@@ -1151,7 +1190,7 @@ __device__ __forceinline__ bool rhs_mbar_wait(uint32_t mbar, uint32_t parity, vo
 template <typename T, int D, int N, int DZ, int DY, int NTH, int MINB, int FLUX, bool TMA = false>
 __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__ Us, const T* U0,
                                              T* Uout, T* __restrict__ faces,
-                                             int stage, int one_slot, int fuse_restrict,
+                                             int stage, int one_slot, int flags,
                                              const __grid_constant__ CUtensorMap tmap) {
     constexpr bool CEN = FLUX == AMR_FLUX_CENTRAL;
     constexpr int EXT = CEN ? 2 : 0;                   // central: faces i - 3/2 .. N + 1/2 along d
@@ -1163,6 +1202,8 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
     constexpr int CPT = (C::CELLS + NTH - 1) / NTH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
+    // the step's last stage moves the time on: nothing after it in the step reads it
+    if ((flags & RHS_ADVANCE) && blockIdx.x == 0 && threadIdx.x == 0) g.time->t = g.time->t + g.time->dt;
     unsigned char* sbase = smem_raw;
     if constexpr (TMA)                                   // tensor-copy destinations: 128-byte aligned
         sbase += (128u - (rhs_smem_addr(smem_raw) & 127u)) & 127u;
@@ -1197,7 +1238,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
         const int slot = one_slot >= 0 ? one_slot : g.leaf_list[pi];
         const int lev = g.level[slot];
         const int pf = g.pflag[slot];
-        const bool fuse = fuse_restrict && lev == g.L - 1 && lev >= 1;
+        const bool fuse = (flags & RHS_RESTRICT) && lev == g.L - 1 && lev >= 1;
         // 1. stage the chunk and its halo as primitives, loading 16-byte vectors
         //    along x (slot rows are 16-byte aligned)
         {
@@ -1747,12 +1788,13 @@ __global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int o
 }
 
 // ---------------------------------------------------------------------------
-// K7: CFL reduction over leaf cells: lambda = sum_d (|u_d| + c) / dx_d in FP64,
+// K7: CFL reduction over leaf cells (finalize: and the step that follows from
+// it, set by the grid's last block): lambda = sum_d (|u_d| + c) / dx_d in FP64,
 // c = sqrt(gamma p / rho); block max by warp shuffles, grid max by atomicMax
 // on the bit pattern (valid for non-negative doubles)
 // ---------------------------------------------------------------------------
 template <typename T, int D, int N>
-__global__ void __launch_bounds__(256) k_cfl(Grid g, const T* U, int one_slot) {
+__global__ void __launch_bounds__(256) k_cfl(Grid g, const T* U, int one_slot, int finalize) {
     // the running maximum is kept in the storage precision (exact: the
     // maximum of FP32 values converts to the maximum of their FP64 images)
     // and turned into FP64 once per CTA. A work item is VE consecutive
@@ -1812,7 +1854,16 @@ __global__ void __launch_bounds__(256) k_cfl(Grid g, const T* U, int one_slot) {
         double m = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) atomicMax(&g.time->lam, (unsigned long long)__double_as_longlong(m));
+        if (lane == 0) {
+            atomicMax(&g.time->lam, (unsigned long long)__double_as_longlong(m));
+            if (finalize) {                              // the last block of the grid sets the step
+                __threadfence();
+                if (atomicAdd(&g.time->ticket, 1u) == gridDim.x - 1) {
+                    g.time->ticket = 0u;
+                    finalize_dt(g.time, atomicMax(&g.time->lam, 0ull), g.cfl, g.t_end);
+                }
+            }
+        }
     }
 }
 
@@ -2043,7 +2094,7 @@ __global__ void __launch_bounds__(256) k_prolong_new(Grid g, T* U, const int* li
         for (int ci = threadIdx.x; ci < NC; ci += blockDim.x) {
             int l[3] = {ci % N, D >= 2 ? (ci / N) % N : 0, D == 3 ? ci / (N * N) : 0};
             T val[NV];
-            prolong_cell<T, D, N, false>(g, U, m, l, val);
+            prolong_cell<T, D, N, false>(g, U, m, l, BcState{0.0, nullptr, nullptr}, val);
             const int sx = l[0] + G, sy = D >= 2 ? l[1] + G : 0, sz = D == 3 ? l[2] + G : 0;
 #pragma unroll
             for (int v = 0; v < NV; ++v) U[slot_index(g, slot, v, sz, sy, sx)] = val[v];

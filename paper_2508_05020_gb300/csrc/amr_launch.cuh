@@ -126,47 +126,47 @@ inline double4 d4(const double* v) { return make_double4(v[0], v[1], v[2], v[3])
 
 template <typename T, int D, int N, int FLUX, int V>
 static cudaError_t rhs_launch_v(const Grid& g, const T* Us, const T* U0, T* Uout, T* faces, int stage, int grid,
-                                cudaStream_t s, int one_slot, int fuse, const CUtensorMap* tmap) {
+                                cudaStream_t s, int one_slot, int flags, const CUtensorMap* tmap) {
     using C = RhsCfg<T, D, N, V>;
     static const CUtensorMap none{};                     // the kernels without tensor copies ignore it
     if (C::TMA && !tmap) return cudaErrorInvalidValue;   // no tensor map of this state array
     k_rhs<T, D, N, C::DZ, C::DY, C::NTH, C::MINB, FLUX, C::TMA>
         <<<grid, C::NTH, rhs_smem_bytes<T, D, N, C::DZ, C::DY, FLUX, C::TMA>(), s>>>(g, Us, U0, Uout, faces, stage,
-                                                                          one_slot, fuse, tmap ? *tmap : none);
+                                                                          one_slot, flags, tmap ? *tmap : none);
     return cudaSuccess;
 }
 
 template <typename T, int D, int N, int FLUX>
 static cudaError_t rhs_launch_f(const Grid& g, const T* Us, const T* U0, T* Uout, T* faces, int stage, int grid,
-                                cudaStream_t s, int one_slot, int fuse, const CUtensorMap* tmap, int cls) {
+                                cudaStream_t s, int one_slot, int flags, const CUtensorMap* tmap, int cls) {
     if constexpr (D >= 2)
         if (cls == RHS_FEW && g.rhs_shape == 0)
-            return rhs_launch_v<T, D, N, FLUX, FEW>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap);
+            return rhs_launch_v<T, D, N, FLUX, FEW>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap);
     if constexpr (RhsShapes<T, D, N, FLUX>::n == 5) {
         switch (g.rhs_shape) {
-        case 1: return rhs_launch_v<T, D, N, FLUX, 1>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap);
-        case 2: return rhs_launch_v<T, D, N, FLUX, 2>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap);
-        case 3: return rhs_launch_v<T, D, N, FLUX, 3>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap);
-        case 4: return rhs_launch_v<T, D, N, FLUX, 4>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap);
+        case 1: return rhs_launch_v<T, D, N, FLUX, 1>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap);
+        case 2: return rhs_launch_v<T, D, N, FLUX, 2>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap);
+        case 3: return rhs_launch_v<T, D, N, FLUX, 3>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap);
+        case 4: return rhs_launch_v<T, D, N, FLUX, 4>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap);
         default: break;
         }
     }
-    return rhs_launch_v<T, D, N, FLUX, 0>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap);
+    return rhs_launch_v<T, D, N, FLUX, 0>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap);
 }
 
 template <typename T, int D, int N>
 static cudaError_t rhs_launch(const Grid& g, const T* Us, const T* U0, T* Uout, T* faces, int stage, int grid,
-                              cudaStream_t s, int one_slot, int fuse, const CUtensorMap* tmap, int cls) {
+                              cudaStream_t s, int one_slot, int flags, const CUtensorMap* tmap, int cls) {
     // one instantiation per flux: the Rusanov kernel carries no HLLC code
     cudaError_t e;
     if (g.flux == AMR_FLUX_CENTRAL)
-        e = rhs_launch_f<T, D, N, AMR_FLUX_CENTRAL>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap, cls);
+        e = rhs_launch_f<T, D, N, AMR_FLUX_CENTRAL>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap, cls);
     else if (g.flux == AMR_FLUX_HYBRID)
-        e = rhs_launch_f<T, D, N, AMR_FLUX_HYBRID>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap, cls);
+        e = rhs_launch_f<T, D, N, AMR_FLUX_HYBRID>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap, cls);
     else if (g.flux == AMR_FLUX_HLLC)
-        e = rhs_launch_f<T, D, N, AMR_FLUX_HLLC>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap, cls);
+        e = rhs_launch_f<T, D, N, AMR_FLUX_HLLC>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap, cls);
     else
-        e = rhs_launch_f<T, D, N, AMR_FLUX_RUSANOV>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse, tmap, cls);
+        e = rhs_launch_f<T, D, N, AMR_FLUX_RUSANOV>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags, tmap, cls);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -266,15 +266,15 @@ cudaError_t Kernels<T>::prepare(const Grid& g) {
 }
 
 template <typename T>
-cudaError_t Kernels<T>::ghost_fill(const Grid& g, T* U, int level, double tfrac, int grid, cudaStream_t s,
-                                   int one_slot, int chunk, bool stage_only) {
+cudaError_t Kernels<T>::ghost_fill(const Grid& g, T* U, double tfrac, int grid, cudaStream_t s, int one_slot,
+                                   int chunk, bool stage_only) {
     if (chunk < 32) return cudaErrorInvalidValue;
     const int n_cells = stage_only ? g.n_ghost_face : g.n_ghost;
     if (stage_only) {
-        AMR_DISPATCH(g, (k_ghost<T, D, N, true><<<grid, 256, 0, s>>>(g, U, level, tfrac, one_slot, d4(g.dmr_pre),
+        AMR_DISPATCH(g, (k_ghost<T, D, N, true><<<grid, 256, 0, s>>>(g, U, tfrac, one_slot, d4(g.dmr_pre),
                                                                       d4(g.dmr_post), chunk, n_cells)));
     } else {
-        AMR_DISPATCH(g, (k_ghost<T, D, N, false><<<grid, 256, 0, s>>>(g, U, level, tfrac, one_slot, d4(g.dmr_pre),
+        AMR_DISPATCH(g, (k_ghost<T, D, N, false><<<grid, 256, 0, s>>>(g, U, tfrac, one_slot, d4(g.dmr_pre),
                                                                        d4(g.dmr_post), chunk, n_cells)));
     }
     return cudaGetLastError();
@@ -282,8 +282,8 @@ cudaError_t Kernels<T>::ghost_fill(const Grid& g, T* U, int level, double tfrac,
 
 template <typename T>
 cudaError_t Kernels<T>::rhs_stage(const Grid& g, const T* Us, const T* U0, T* Uout, T* faces, int stage, int grid,
-                                  cudaStream_t s, int one_slot, int fuse_restrict, const void* tmap, int cls) {
-    AMR_DISPATCH(g, return (rhs_launch<T, D, N>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, fuse_restrict,
+                                  cudaStream_t s, int one_slot, int flags, const void* tmap, int cls) {
+    AMR_DISPATCH(g, return (rhs_launch<T, D, N>(g, Us, U0, Uout, faces, stage, grid, s, one_slot, flags,
                                                 static_cast<const CUtensorMap*>(tmap), cls)));
     return cudaSuccess;
 }
@@ -302,8 +302,8 @@ cudaError_t Kernels<T>::restrict_level(const Grid& g, T* U, int level, int grid,
 }
 
 template <typename T>
-cudaError_t Kernels<T>::cfl(const Grid& g, const T* U, int grid, cudaStream_t s, int one_slot) {
-    AMR_DISPATCH(g, (k_cfl<T, D, N><<<grid, 256, 0, s>>>(g, U, one_slot)));
+cudaError_t Kernels<T>::cfl(const Grid& g, const T* U, int grid, cudaStream_t s, int one_slot, bool finalize) {
+    AMR_DISPATCH(g, (k_cfl<T, D, N><<<grid, 256, 0, s>>>(g, U, one_slot, finalize ? 1 : 0)));
     return cudaGetLastError();
 }
 
