@@ -1661,71 +1661,98 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
 // the mean F_f of the 2^(d-1) fine face fluxes (summed in lexicographic
 // z, y, x order, times 2^-(d-1)), applied to the stage result as
 // U -/+ b dt (F_f - F_c) / dx on the high/low face; faces x-, x+, y-, ... in turn.
+// A thread takes a boundary cell and applies all its faces' corrections to it
+// (a cell at an edge or corner has two or three), so the faces of a patch need
+// no barrier between them and a patch costs one round of loads, not one per
+// face: the kernel waits on loads (it moves a few hundred kilobytes). A step
+// with 854 leaves of 8^3 (FP32): 312 -> 270 us, with 760 leaves of 16^2: 120 -> 105.
 // ---------------------------------------------------------------------------
+template <typename T, int D, int N>
+__device__ __forceinline__ void reflux_patch(const Grid& g, T* Uout, const T* __restrict__ faces, T rb, T dt, int e) {
+    constexpr int NV = D + 2;
+    constexpr int TRANS = Chunk<D, N, 1, N>::TRANS;
+    const int slot = g.reflux_list[e];
+    const int lev = g.level[slot];
+    const int* fine = g.reflux_fine + (long long)e * 24;
+    unsigned active = 0;
+#pragma unroll
+    for (int f = 0; f < 2 * D; ++f) active |= fine[f * 4] >= 0 ? 1u << f : 0u;
+    for (int i = threadIdx.x; i < 2 * D * TRANS; i += blockDim.x) {
+        const int f = i / TRANS, t = i - f * TRANS;
+        if (!(active >> f & 1)) continue;
+        const int fd = f >> 1;
+        const int th = D == 3 ? t / N : 0, tl = D == 1 ? 0 : (D == 3 ? t % N : t);
+        const int edge = (f & 1) ? N - 1 : 0;
+        // transverse coordinates in (z, y, x) order, the higher dimension first
+        const int cx = fd == 0 ? edge : tl;
+        const int cy = fd == 1 ? edge : (D == 3 && fd == 2 ? th : tl);
+        const int cz = fd == 2 ? edge : th;
+        const int cell[3] = {cx, cy, cz};
+        // the cell belongs to the first of its faces that is corrected
+        bool mine = true;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const int side = cell[d] == 0 ? 0 : (cell[d] == N - 1 ? 1 : -1);
+            if (d < fd && side >= 0 && (active >> (2 * d + side) & 1)) mine = false;
+        }
+        if (!mine) continue;
+        const long long id = slot_index(g, slot, 0, D == 3 ? cz + G : 0, D >= 2 ? cy + G : 0, cx + G);
+        T u[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) u[v] = Uout[id + v * g.slot_elems];
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const int side = cell[d] == 0 ? 0 : (cell[d] == N - 1 ? 1 : -1);
+            if (d < fd || side < 0 || !(active >> (2 * d + side) & 1)) continue;
+            const int* fs = fine + (2 * d + side) * 4;
+            const int hi = D == 3 ? (d == 2 ? cy : cz) : 0;
+            const int lo = D == 1 ? 0 : (d == 0 ? cy : cx);
+            const T dx = T(g.dx[lev][d]);
+            const T* src[1 << (D - 1)];                  // the fine faces' first variable
+            bool whole = true;
+#pragma unroll
+            for (int k = 0; k < (1 << (D - 1)); ++k) {
+                const int fh = 2 * hi + (D == 3 ? k >> 1 : 0), fl = 2 * lo + (D >= 2 ? k & 1 : 0);
+                const int fslot = D == 3 ? fs[fh / N * 2 + fl / N] : (D == 2 ? fs[fl / N] : fs[0]);
+                const int fidx = D == 3 ? fh % N * N + fl % N : (D == 2 ? fl % N : 0);
+                whole = whole && fslot >= 0;
+                src[k] = faces + ((long long)(fslot < 0 ? slot : fslot) * 2 * D + 2 * d + (1 - side)) * NV * TRANS + fidx;
+            }
+            if (!whole) {                                // inconsistent table: report, skip
+                atomicOr(&g.time->err, ERR_MESH);
+                continue;
+            }
+            const T* Fc = faces + ((long long)slot * 2 * D + 2 * d + side) * NV * TRANS + (D == 1 ? 0 : (D == 2 ? lo : hi * N + lo));
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                T acc = src[0][v * TRANS];
+#pragma unroll
+                for (int k = 1; k < (1 << (D - 1)); ++k) acc = acc + src[k][v * TRANS];
+                const T Ff = acc * T(D == 3 ? 0.25 : (D == 2 ? 0.5 : 1.0));
+                const T df = Ff - Fc[v * TRANS];
+                const T diff = sizeof(T) == 8 && exact_reciprocal(dx) ? df * (T(1) / dx) : Num<T>::div(df, dx);
+                u[v] = side ? u[v] - rb * (dt * diff) : u[v] + rb * (dt * diff);
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Uout[id + v * g.slot_elems] = u[v];
+    }
+}
+
+// b of a stage: its share of dt R in the result
+template <typename T>
+__device__ __forceinline__ T stage_b(int stage) {
+    return stage == 0 ? T(1) : (stage == 1 ? T(0.25) : T(2.0 / 3.0));
+}
+
 template <typename T, int D, int N>
 __global__ void __launch_bounds__(256) k_reflux(Grid g, T* Uout, const T* __restrict__ faces, int stage,
                                                 int one_item) {
-    constexpr int NV = D + 2;
-    constexpr int TRANS = Chunk<D, N, 1, N>::TRANS;
     if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
-    const T rb = stage == 0 ? T(1) : (stage == 1 ? T(0.25) : T(2.0 / 3.0));
     const T dt = T(g.time->dt);
     const int n = one_item >= 0 ? one_item + 1 : g.counts[2];
-    for (int e = one_item >= 0 ? one_item : blockIdx.x; e < n; e += gridDim.x) {
-        const int slot = g.reflux_list[e];
-        const int lev = g.level[slot];
-        for (int d = 0; d < D; ++d) {
-            for (int side = 0; side < 2; ++side) {
-                const int* fs = g.reflux_fine + ((long long)e * 6 + 2 * d + side) * 4;
-                if (fs[0] < 0) continue;
-                const T dx = T(g.dx[lev][d]);
-                for (int t = threadIdx.x; t < TRANS; t += blockDim.x) {
-                    const int th = D == 3 ? t / N : 0;       // transverse (hi, lo) in (z, y, x) order
-                    const int tl = D == 1 ? 0 : (D == 3 ? t % N : t);
-                    int cell[3] = {0, 0, 0};
-                    cell[d] = side ? N - 1 : 0;
-                    {
-                        int j = 0;
-                        for (int e2 = D - 1; e2 >= 0; --e2) {   // hi transverse first
-                            if (e2 == d) continue;
-                            cell[e2] = (D == 3 && j == 0) ? th : tl;
-                            ++j;
-                        }
-                    }
-                    const int sx = cell[0] + G, sy = D >= 2 ? cell[1] + G : 0, sz = D == 3 ? cell[2] + G : 0;
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        T acc = T(0);
-                        bool first = true;
-                        for (int ah = 0; ah < (D == 3 ? 2 : 1); ++ah) {
-                            for (int al = 0; al < (D >= 2 ? 2 : 1); ++al) {
-                                const int fh = 2 * th + ah, fl = 2 * tl + al;
-                                const int ph = fh / N, pl = fl / N;
-                                const int lh = fh % N, ll = fl % N;
-                                const int fslot = D == 3 ? fs[ph * 2 + pl] : (D == 2 ? fs[pl] : fs[0]);
-                                const int fidx = D == 3 ? lh * N + ll : (D == 2 ? ll : 0);
-                                if (fslot < 0) {             // inconsistent table: report, skip
-                                    atomicOr(&g.time->err, ERR_MESH);
-                                    continue;
-                                }
-                                const T val = faces[((long long)fslot * 2 * D + 2 * d + (1 - side)) * NV * TRANS +
-                                                    v * TRANS + fidx];
-                                acc = first ? val : acc + val;
-                                first = false;
-                            }
-                        }
-                        const T Ff = acc * T(D == 3 ? 0.25 : (D == 2 ? 0.5 : 1.0));
-                        const T Fc = faces[((long long)slot * 2 * D + 2 * d + side) * NV * TRANS + v * TRANS + t];
-                        const T diff = Num<T>::div(Ff - Fc, dx);
-                        const long long id = slot_index(g, slot, v, sz, sy, sx);
-                        const T u = Uout[id];
-                        Uout[id] = side ? u - rb * (dt * diff) : u + rb * (dt * diff);
-                    }
-                }
-                __syncthreads();
-            }
-        }
-    }
+    for (int e = one_item >= 0 ? one_item : blockIdx.x; e < n; e += gridDim.x)
+        reflux_patch<T, D, N>(g, Uout, faces, stage_b<T>(stage), dt, e);
 }
 
 // ---------------------------------------------------------------------------
