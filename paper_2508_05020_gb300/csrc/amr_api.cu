@@ -413,6 +413,9 @@ long long patch_cells(const amr_ctx* c) {
 }
 long long cfl_threads(const amr_ctx* c) { return patch_cells(c) * (c->precision / 8) / 16; }
 long long restrict_threads(const amr_ctx* c) { return patch_cells(c) >> c->dim; }
+// the reflux, restriction and next ghost fill of a stage as one launch: 1D, up
+// to 127 patches (see k_after)
+bool after_in_one(const amr_ctx* c) { return c->dim == 1 && size_bits(c) <= 7; }
 
 // class and grid of the fused RHS for the present hierarchy
 template <typename T>
@@ -512,11 +515,12 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
     const int gghost = grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, true));
     const int greflux = grid_for(c, c->tune[AMR_TUNE_REFLUX_GRID], 256);
     const int grestrict = grid_for(c, c->tune[AMR_TUNE_RESTRICT_GRID], restrict_threads(c));
+    const bool after = !c->timing && after_in_one(c);
     for (int s = 0; s < 3; ++s) {
         T* src = St<T>(c, s == 0 ? 0 : s);
         T* dst = St<T>(c, s == 0 ? 1 : (s == 1 ? 2 : 0));
         CK(mark(c->ev[s][0]), "event");
-        if (!(s == 0 && skip_fill0)) {
+        if (s == 0 ? !skip_fill0 : !after) {
             CK(Kernels<T>::ghost_fill(g, src, tfrac[s], gghost, c->stream, -1, c->tune[AMR_TUNE_GHOST_CHUNK], true),
                "ghost fill");
             ++k;
@@ -527,6 +531,15 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
            "rhs stage");
         CK(mark(c->ev[s][2]), "event");
         ++k;
+        if (after) {
+            if (c->L > 1 || s < 2) {
+                CK(Kernels<T>::after_stage(g, dst, reinterpret_cast<T*>(c->faces), s, s < 2, s < 2 ? tfrac[s + 1] : 0.0,
+                                           c->tune[AMR_TUNE_GHOST_CHUNK], c->stream),
+                   "after stage");
+                ++k;
+            }
+            continue;
+        }
         if (c->L > 1) {
             CK(Kernels<T>::reflux(g, dst, reinterpret_cast<T*>(c->faces), s, greflux, c->stream, -1), "reflux");
             ++k;

@@ -157,6 +157,10 @@ struct Kernels {
     // covered cells of level-1 patches from the children of level `level`
     static cudaError_t restrict_level(const Grid& g, T* U, int level, int grid, cudaStream_t s,
                                       int one_slot);
+    // reflux, the restriction of levels L - 2 .. 1 and (next) the next stage's
+    // ghost fill of U in one launch, for a small 1D hierarchy
+    static cudaError_t after_stage(const Grid& g, T* U, const T* faces, int stage, bool next, double tfrac, int chunk,
+                                   cudaStream_t s);
     // finalize: the step too, as launch_finalize_dt sets it
     static cudaError_t cfl(const Grid& g, const T* U, int grid, cudaStream_t s, int one_slot, bool finalize = false);
     static cudaError_t init_ic(const Grid& g, T* U, const int* list, int n, cudaStream_t s);

@@ -954,14 +954,11 @@ __device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* 
 // shared-memory copy; warps never wait for one another.
 // ---------------------------------------------------------------------------
 template <typename T, int D, int N, bool STAGE>
-__global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(Grid g, T* U, double tfrac, int one_slot,
-                                               double4 pre, double4 post, int chunk, int n_cells) {
+__device__ __forceinline__ void ghost_items(const Grid& g, T* U, double tfrac, int one_slot, double4 pre, double4 post,
+                                            int chunk, int n_cells, int warp, int nw, PatchMeta& m) {
     constexpr bool stage_only = STAGE;                  // compiled apart: the full fill keeps its registers
     constexpr int NV = D + 2;
-    __shared__ PatchMeta metas[256 / 32];
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    PatchMeta& m = metas[warp];
+    const int lane = threadIdx.x & 31;
     const int npatch = one_slot >= 0 ? 1 : g.counts[0];
     const double pr[4] = {pre.x, pre.y, pre.z, pre.w};
     const double po[4] = {post.x, post.y, post.z, post.w};
@@ -973,8 +970,7 @@ __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(
     const int span = stage_only ? BOX : n_cells;          // table entries one run of items covers
     const int nruns = stage_only ? 2 * D : 1;
     const int nchunk = (span + chunk - 1) / chunk;        // chunk: ghost cells per work item
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int item = blockIdx.x * (blockDim.x >> 5) + warp; item < npatch * nruns * nchunk; item += nw) {
+    for (int item = warp; item < npatch * nruns * nchunk; item += nw) {
         const int pi = item / (nruns * nchunk);
         const int rest = item - pi * nruns * nchunk;
         const int run = rest / nchunk;
@@ -1060,6 +1056,16 @@ __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(
         }
         __syncwarp();                                    // the copy is read until here
     }
+}
+
+template <typename T, int D, int N, bool STAGE>
+__global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(Grid g, T* U, double tfrac, int one_slot,
+                                               double4 pre, double4 post, int chunk, int n_cells) {
+    __shared__ PatchMeta metas[256 / 32];
+    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
+    const int warp = threadIdx.x >> 5;
+    ghost_items<T, D, N, STAGE>(g, U, tfrac, one_slot, pre, post, chunk, n_cells, blockIdx.x * (256 / 32) + warp,
+                                gridDim.x * (256 / 32), metas[warp]);
 }
 
 // Restriction mean of the 2^d children of a covered coarse cell, given in
@@ -1761,7 +1767,8 @@ __global__ void __launch_bounds__(256) k_reflux(Grid g, T* Uout, const T* __rest
 // summed in FP64 (FP32 fields: an error-free FP32 pair sum, rounded once)
 // ---------------------------------------------------------------------------
 template <typename T, int D, int N>
-__global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int one_slot) {
+__device__ __forceinline__ void restrict_items(const Grid& g, T* U, int level, int one_slot, long long thread,
+                                               long long nthreads) {
     // thread <-> CP coarse cells adjacent in x (FP32: 2, FP64: 1), whose
     // children of each (y, z) offset are VE consecutive fine cells of a row:
     // one aligned 16-byte vector (interior rows start on a 32-byte boundary)
@@ -1772,12 +1779,10 @@ __global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int o
     constexpr int HC = (D == 1 ? H : (D == 2 ? H * H : H * H * H)) / CP;
     constexpr int NYZ = 1 << (D - 1);                    // child (y, z) offsets
     constexpr int NCH = 1 << D;
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
     const int lo = g.level_off[level], hi = g.level_off[level + 1];
     const int npatch = one_slot >= 0 ? 1 : hi - lo;
     const long long total = (long long)npatch * HC;
-    for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < total;
-         it += (long long)gridDim.x * blockDim.x) {
+    for (long long it = thread; it < total; it += nthreads) {
         const int pi = (int)(it / HC);
         const int ci = (int)(it - (long long)pi * HC);
         const int slot = one_slot >= 0 ? one_slot : g.all_list[lo + pi];
@@ -1812,6 +1817,49 @@ __global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int o
                 U[slot_index(g, par, v, D == 3 ? oz + cz + G : 0, D >= 2 ? oy + cy + G : 0, ox + cx + q + G)] = mean;
             }
     }
+}
+
+template <typename T, int D, int N>
+__global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int one_slot) {
+    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
+    restrict_items<T, D, N>(g, U, level, one_slot, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
+}
+
+// ---------------------------------------------------------------------------
+// What follows the RHS of a stage, for a small 1D hierarchy, in one launch of one
+// cluster: the flux correction, the restriction level by level and the next
+// stage's ghost fill, with the cluster's barrier where a launch
+// would lie. Eight SMs suffice while each part is a round or two of loads: us
+// per step in FP32, separate launches / this one, 28 patches 49.5 / 43.4, 76
+// patches 49.5 / 45.4, 264 patches 49.5 / 51.5. In 2D and 3D the parts are too
+// large for them from the smallest meshes on (64 patches of 8^2: 54.6 / 60.7).
+// ---------------------------------------------------------------------------
+constexpr int AFTER_CTAS = 8;
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+// next: the next stage's ghosts are filled, at time t + tfrac dt
+template <typename T, int D, int N>
+__global__ void __cluster_dims__(AFTER_CTAS, 1, 1) __launch_bounds__(256)
+    k_after(Grid g, T* U, const T* __restrict__ faces, int stage, int next, double tfrac, double4 pre, double4 post,
+            int chunk, int n_cells) {
+    __shared__ PatchMeta metas[256 / 32];
+    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
+    const T dt = T(g.time->dt);
+    for (int e = blockIdx.x; e < g.counts[2]; e += AFTER_CTAS)
+        reflux_patch<T, D, N>(g, U, faces, stage_b<T>(stage), dt, e);
+    for (int l = g.L - 2; l >= 1; --l) {                 // level L - 1: fused into the RHS
+        cluster_barrier();
+        restrict_items<T, D, N>(g, U, l, -1, blockIdx.x * 256 + threadIdx.x, AFTER_CTAS * 256);
+    }
+    if (!next) return;
+    cluster_barrier();
+    const int warp = threadIdx.x >> 5;
+    ghost_items<T, D, N, true>(g, U, tfrac, -1, pre, post, chunk, n_cells, blockIdx.x * (256 / 32) + warp,
+                               AFTER_CTAS * (256 / 32), metas[warp]);
 }
 
 // ---------------------------------------------------------------------------

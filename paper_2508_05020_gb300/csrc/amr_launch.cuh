@@ -302,6 +302,21 @@ cudaError_t Kernels<T>::restrict_level(const Grid& g, T* U, int level, int grid,
 }
 
 template <typename T>
+cudaError_t Kernels<T>::after_stage(const Grid& g, T* U, const T* faces, int stage, bool next, double tfrac, int chunk,
+                                    cudaStream_t s) {
+    auto go = [&](auto n) {
+        k_after<T, 1, decltype(n)::value><<<AFTER_CTAS, 256, 0, s>>>(g, U, faces, stage, next ? 1 : 0, tfrac, d4(g.dmr_pre),
+                                                                     d4(g.dmr_post), chunk, g.n_ghost_face);
+    };
+    if (g.dim != 1) return cudaErrorInvalidValue;
+    if (g.N == 8) go(std::integral_constant<int, 8>{});
+    else if (g.N == 16) go(std::integral_constant<int, 16>{});
+    else if (g.N == 32) go(std::integral_constant<int, 32>{});
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t Kernels<T>::cfl(const Grid& g, const T* U, int grid, cudaStream_t s, int one_slot, bool finalize) {
     AMR_DISPATCH(g, (k_cfl<T, D, N><<<grid, 256, 0, s>>>(g, U, one_slot, finalize ? 1 : 0)));
     return cudaGetLastError();
