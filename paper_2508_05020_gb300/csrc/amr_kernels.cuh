@@ -339,6 +339,11 @@ __device__ __forceinline__ void weno5_lr(const T (&w)[6], T& left, T& right, boo
 // normal momentum, tangential momenta, energy).
 // ---------------------------------------------------------------------------
 template <typename T, int NT, int FLUX>
+__device__ __forceinline__ void flux_of_values(const T (&wl)[NT + 3], const T (&wr)[NT + 3], const T (&p)[6],
+                                               const T (&un)[6], const T (&ut)[NT > 0 ? NT : 1][6], const T (&Tt)[6],
+                                               T z, T kap, T gamma, T gm1, T (&F)[NT + 3]);
+
+template <typename T, int NT, int FLUX>
 __device__ __forceinline__ void face_flux(const T (&p)[6], const T (&un)[6], const T (&ut)[NT > 0 ? NT : 1][6],
                                           const T (&Tt)[6], T gamma, T gm1, T (&F)[NT + 3]) {
     constexpr int NF = NT + 3;
@@ -371,6 +376,15 @@ __device__ __forceinline__ void face_flux(const T (&p)[6], const T (&un)[6], con
     if (!interpolate(std::true_type{})) {
         if constexpr (sizeof(T) == 4) interpolate(std::false_type{});
     }
+    flux_of_values<T, NT, FLUX>(wl, wr, p, un, ut, Tt, z, kap, gamma, gm1, F);
+}
+
+// the rest of face_flux: the flux from the left and right characteristic values
+template <typename T, int NT, int FLUX>
+__device__ __forceinline__ void flux_of_values(const T (&wl)[NT + 3], const T (&wr)[NT + 3], const T (&p)[6],
+                                               const T (&un)[6], const T (&ut)[NT > 0 ? NT : 1][6], const T (&Tt)[6],
+                                               T z, T kap, T gamma, T gm1, T (&F)[NT + 3]) {
+    constexpr int NF = NT + 3;
     const T z2 = T(2) * z;
     T pL = T(0.5) * (wl[0] + wl[NF - 1]);
     T unL = Num<T>::div(wl[NF - 1] - wl[0], z2);
@@ -1145,11 +1159,22 @@ template <int D, int N, int DZ, int DY, int EXT = 0, bool PADQ = false> struct C
     static constexpr int TRANS = D == 1 ? 1 : (D == 2 ? N : N * N);   // cells on a patch face
 };
 
+// FP64 in 1D: the six WENO values of a face are computed by six threads. A patch
+// has only N + 1 faces, and a sub-partition issues one FP64 warp instruction
+// in 31 ns however few of its lanes are in use, so the time of a patch is the
+// longest chain of one thread: 112 + 57 instructions instead of 640. A step of
+// the shock tube (8 leaves): 143 -> 105 us; 1024 leaves: 328 -> 197 us.
+template <typename T, int D, int FLUX>
+constexpr bool rhs_splits_faces = D == 1 && sizeof(T) == 8 && (FLUX == AMR_FLUX_RUSANOV || FLUX == AMR_FLUX_HLLC);
+
 template <typename T, int D, int N, int DZ, int DY, int FLUX, bool TMA = false>
 constexpr size_t rhs_smem_bytes() {
     using C = Chunk<D, N, DZ, DY, FLUX == AMR_FLUX_CENTRAL ? 2 : 0, TMA>;
-    // TMA: 128 bytes to align the base, an mbarrier and an abort word
-    return sizeof(T) * ((size_t)(D + 2) * C::QN + (size_t)(D + 2) * C::FMAX) + (TMA ? 128 + 16 : 0);
+    // TMA: 128 bytes to align the base, an mbarrier and an abort word; split
+    // faces: the six characteristic values, z and kappa of each
+    return sizeof(T) * ((size_t)(D + 2) * C::QN + (size_t)(D + 2) * C::FMAX +
+                        (rhs_splits_faces<T, D, FLUX> ? 8 * (N + 1) : 0)) +
+           (TMA ? 128 + 16 : 0);
 }
 
 // Tensor copies (TMA) of the halo planes: a 4D tiled load of a box into
@@ -1184,6 +1209,98 @@ __device__ __forceinline__ bool rhs_mbar_wait(uint32_t mbar, uint32_t parity, vo
         if ((it & 63u) == 63u && clock64() - t0 > TC_WAIT_CYCLES) {
             *abort = 1;
             return false;
+        }
+    }
+}
+
+// The faces of a 1D FP64 patch from its staged primitives q (p, u, T), each by
+// six threads and then two: Fs receives the fluxes, W is scratch for 8 (N + 1)
+// values, save(f, F) sees every flux once. Bit for bit the arithmetic of face_flux.
+template <int N, int NTH, int FLUX, class Save>
+__device__ __forceinline__ void split_faces(const double* q, int qn, double* Fs, int fstride, double* W, double gamma,
+                                            double gm1, Save save) {
+    constexpr int NF1 = N + 1;
+    double* Z = W + 6 * NF1;
+    double* K = Z + NF1;
+    for (int e = threadIdx.x; e < 6 * NF1; e += NTH) {
+        const int w = e / NF1, f = e - w * NF1, field = w % 3, right = w / 3;
+        const double* p = q + f;                          // nodes f .. f + 5
+        const double* u = q + qn + f;
+        const double* Tt = q + 2 * qn + f;
+        const double rbar = (0.5 * (p[2] + p[3])) / (0.5 * (Tt[2] + Tt[3]));
+        const double cbar = sqrt(gamma * (0.5 * (Tt[2] + Tt[3])));
+        const double z = rbar * cbar;
+        const double kap = gm1 / (gamma * rbar);
+        if (w == 0) {
+            Z[f] = z;
+            K[f] = kap;
+        }
+        // w1 = p - z u, w2 = T - kappa p, w5 = p + z u
+        const double* A = field == 1 ? Tt : p;
+        const double* B = field == 1 ? p : u;
+        const double c = field == 0 ? -z : (field == 1 ? -kap : z);
+        double v[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const int n = right ? 5 - k : k;
+            v[k] = A[n] + c * B[n];
+        }
+        W[e] = weno5_side(v[0], v[1], v[2], v[3], v[4], 3.0 * v[2], 3.0 * v[3]);
+    }
+    __syncthreads();
+    if constexpr (FLUX == AMR_FLUX_RUSANOV) {
+        // two lanes per face, one for each side; both ends of a pair are in one warp
+        for (int i = threadIdx.x; i < (2 * NF1 + 31) / 32 * 32; i += NTH) {
+            const int f = i >> 1 < N ? i >> 1 : N, right = i & 1;
+            const double z = Z[f], kap = K[f];
+            const double* w = W + right * 3 * NF1 + f;
+            double p = 0.5 * (w[0] + w[2 * NF1]);
+            double un = (w[2 * NF1] - w[0]) / (2.0 * z);
+            double Tt = w[NF1] + kap * p;
+            const bool bad = !(p > 0.0) || !(Tt > 0.0);
+            if (__shfl_xor_sync(0xffffffffu, bad ? 1 : 0, 1) || bad) {
+                p = q[f + 2 + right];
+                un = q[qn + f + 2 + right];
+                Tt = q[2 * qn + f + 2 + right];
+            }
+            const double rho = p / Tt;
+            const double c = sqrt(gamma * Tt);
+            const double E = Num<double>::half(rho * (un * un), p / gm1);
+            const double mn = rho * un;
+            const double U[3] = {rho, mn, E}, Fv[3] = {mn, mn * un + p, (E + p) * un};
+            const double s = c + fabs(un);
+            const double so = __shfl_xor_sync(0xffffffffu, s, 1);
+            const double hS = 0.5 * fmax(right ? s : so, right ? so : s);
+            double F[3];
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+                const double Uo = __shfl_xor_sync(0xffffffffu, U[v], 1), Fo = __shfl_xor_sync(0xffffffffu, Fv[v], 1);
+                F[v] = Num<double>::half(Fv[v] + Fo, -(hS * (right ? U[v] - Uo : Uo - U[v])));
+            }
+            if (!right && i >> 1 <= N) {
+#pragma unroll
+                for (int v = 0; v < 3; ++v) Fs[v * fstride + f] = F[v];
+                save(f, F);
+            }
+        }
+    } else {
+        for (int f = threadIdx.x; f <= N; f += NTH) {
+            double p[6], un[6], ut[1][6], Tt[6], wl[3], wr[3], F[3];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                p[k] = q[f + k];
+                un[k] = q[qn + f + k];
+                Tt[k] = q[2 * qn + f + k];
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                wl[k] = W[k * NF1 + f];
+                wr[k] = W[(3 + k) * NF1 + f];
+            }
+            flux_of_values<double, 0, FLUX>(wl, wr, p, un, ut, Tt, Z[f], K[f], gamma, gm1, F);
+#pragma unroll
+            for (int v = 0; v < 3; ++v) Fs[v * fstride + f] = F[v];
+            save(f, F);
         }
     }
 }
@@ -1428,6 +1545,16 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
 #pragma unroll 1
         for (int ph = 0; ph < NPH; ++ph) {
             const int nfp = ph == 0 ? (D >= 2 ? C::F0 + C::F1 : C::F0) : C::F2;
+            if constexpr (rhs_splits_faces<T, D, FLUX>) {
+                split_faces<N, NTH, FLUX>(q, C::QN, Fs, C::FMAX, Fs + NV * C::FMAX, gamma, gm1, [&](int f, const double (&F)[3]) {
+                    const int side = f == 0 ? 0 : (f == N ? 1 : -1);
+                    if (side >= 0 && ((pf >> (8 + side)) & 1)) {
+                        T* dst = faces + ((long long)slot * 2 + side) * NV;
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) dst[v] = F[v];
+                    }
+                });
+            } else
             for (int fp = threadIdx.x; fp < nfp; fp += NTH) {
                 // the face's dimension (uniform across a warp except at the one
                 // x/y boundary of the buffer when F0 is not a multiple of 32).

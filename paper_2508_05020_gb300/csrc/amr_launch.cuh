@@ -37,7 +37,7 @@ template <typename T, int D, int N, int V = 0> struct RhsCfg {
     static constexpr bool F32 = sizeof(T) == 4;
     static constexpr int DZ = D == 3 ? (F32 || N == 8 ? 4 : 2) : 1;
     static constexpr int DY = D == 2 && F32 && N == 32 ? 16 : (D >= 2 && !F32 && N == 16 ? 8 : N);
-    static constexpr int NTH = D == 1 ? 64
+    static constexpr int NTH = D == 1 ? (F32 ? 64 : 128)
                                : D == 2 ? (N == 8 ? (F32 ? 96 : 160) : (F32 || N == 16 ? 128 : 256))
                                         : (N == 8 ? 128 : (F32 ? 256 : 128));
     static constexpr int MINB = D == 1 ? 1
