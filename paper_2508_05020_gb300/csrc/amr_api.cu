@@ -13,7 +13,6 @@
 #include <cstring>
 #include <map>
 #include <new>
-#include <set>
 #include <string>
 #include <unordered_map>
 #include <unordered_set>
@@ -32,6 +31,31 @@ struct Range {
     ~Range() { nvtxRangePop(); }
     Range(const Range&) = delete;
     Range& operator=(const Range&) = delete;
+};
+
+// Free slots as a bit set: the lowest free slot is found from the lowest word
+// that may hold one, without a node per slot.
+struct SlotPool {
+    std::vector<uint64_t> bits;
+    size_t low = 0;                                 // no free slot below 64 low
+    void fill(int n) {                              // slots 0 .. n - 1 free
+        bits.assign(((size_t)n + 63) / 64, ~0ull);
+        if (n & 63) bits.back() = (1ull << (n & 63)) - 1;
+        low = 0;
+    }
+    void insert(int s) {
+        bits[(size_t)s >> 6] |= 1ull << (s & 63);
+        low = std::min(low, (size_t)s >> 6);
+    }
+    int take_lowest() {                             // -1: none
+        for (; low < bits.size(); ++low)
+            if (bits[low]) {
+                const int b = __builtin_ctzll(bits[low]);
+                bits[low] &= bits[low] - 1;
+                return (int)(low * 64) + b;
+            }
+        return -1;
+    }
 };
 
 struct amr_ctx {
@@ -58,7 +82,7 @@ struct amr_ctx {
     int slot_hi = 0;                               // one past the highest slot handed out
     std::vector<uint64_t> key_of;        // slot -> packed key (valid if used)
     std::vector<char> used;
-    std::set<int> free_slots;
+    SlotPool free_slots;
     std::vector<Key> canon;              // canonical patch list
     std::vector<int> canon_slot;
     int level_off_h[MAXL + 1] = {0};
@@ -211,8 +235,14 @@ int slot_lookup(const amr_ctx* c, const Key& k) {
 
 void slot_map_clear(amr_ctx* c) {
     c->slot_of.clear();
-    if (c->mesh.dense()) c->slot_at.assign((size_t)c->mesh.positions(), -1);
-    else c->slot_at.clear();
+    if (!c->mesh.dense()) {
+        c->slot_at.clear();
+    } else if (c->slot_at.size() == (size_t)c->mesh.positions()) {   // only the slots in use have an entry
+        for (int s = 0; s < c->slot_hi; ++s)
+            if (c->used[s]) c->slot_at[(size_t)c->mesh.pos(unpack(c->key_of[s]))] = -1;
+    } else {
+        c->slot_at.assign((size_t)c->mesh.positions(), -1);
+    }
 }
 
 void slot_map_set(amr_ctx* c, const Key& k, int s) {
@@ -262,6 +292,15 @@ void fill_tables(amr_ctx* c, const std::vector<Key>& created) {
         int* nb = h + ml.nbr + (size_t)NBR * s;
         for (int e = 0; e < NBR; ++e) nb[e] = -2;                // offsets in unused dimensions
         const int rz = c->dim == 3 ? 1 : 0, ry = c->dim >= 2 ? 1 : 0;
+        const int ex = m.extent(k.l, 0), ey = m.extent(k.l, 1), ez = m.extent(k.l, 2);
+        if (m.dense() && k.x > 0 && k.x < ex - 1 && (!ry || (k.y > 0 && k.y < ey - 1)) &&
+            (!rz || (k.z > 0 && k.z < ez - 1))) {           // away from the domain's sides: fixed strides
+            const int* p = c->slot_at.data() + m.pos(k);
+            for (int oz = -rz; oz <= rz; ++oz)
+                for (int oy = -ry; oy <= ry; ++oy)
+                    for (int ox = -1; ox <= 1; ++ox)
+                        nb[(oz + 1) * 9 + (oy + 1) * 3 + (ox + 1)] = p[((long long)oz * ey + oy) * ex + ox];
+        } else
         for (int oz = -rz; oz <= rz; ++oz)
             for (int oy = -ry; oy <= ry; ++oy)
                 for (int ox = -1; ox <= 1; ++ox) {
@@ -276,16 +315,22 @@ void fill_tables(amr_ctx* c, const std::vector<Key>& created) {
         // neighbour keeps its face flux for the coarse side
         bool any_ref = false;
         int fine[6][4];
-        for (int f = 0; f < 6; ++f)
-            for (int j = 0; j < 4; ++j) fine[f][j] = -1;       // faces of unused dimensions stay -1 too
+        std::memset(fine, 0xFF, sizeof(fine));                 // -1; faces of unused dimensions stay so
         for (int d = 0; d < c->dim; ++d)
             for (int side = 0; side < 2; ++side) {
+                const int across = nb[13 + (side ? 1 : -1) * (d == 0 ? 1 : (d == 1 ? 3 : 9))];
+                if (across == -2) continue;
+                const bool q_exists = across >= 0;
+                if (!q_exists) {
+                    if (k.l > 0) pf |= 1 << (8 + 2 * d + side);
+                    continue;
+                }
+                if (has_ch || k.l == m.max_level) continue;
                 Key q = k;
                 int* qc[3] = {&q.x, &q.y, &q.z};
                 *qc[d] += side ? 1 : -1;
-                if (!m.wrap(q)) continue;
-                const bool q_exists = m.exists(q);
-                if (!has_ch && q_exists && m.has_children(q)) {
+                m.wrap(q);
+                if (m.has_children(q)) {
                     pf |= 1 << (8 + 2 * d + side);
                     any_ref = true;
                     // children of q adjacent to the face, transverse sub-positions (hi, lo)
@@ -306,7 +351,6 @@ void fill_tables(amr_ctx* c, const std::vector<Key>& created) {
                         fine[2 * d + side][sidx] = slot_lookup(c, f);
                     }
                 }
-                if (k.l > 0 && !q_exists) pf |= 1 << (8 + 2 * d + side);
             }
         h[ml.pflag + s] = pf;
         c->level_off_h[k.l + 1] = (int)i + 1;
@@ -372,10 +416,9 @@ void assign_slots(amr_ctx* c, const std::vector<Key>& created, const std::vector
         else c->slot_of.erase(pack(k));
     }
     std::vector<Key> cr = created;
-    std::sort(cr.begin(), cr.end(), canon_less);
+    if (!std::is_sorted(cr.begin(), cr.end(), canon_less)) std::sort(cr.begin(), cr.end(), canon_less);
     for (const auto& k : cr) {
-        const int s = *c->free_slots.begin();
-        c->free_slots.erase(c->free_slots.begin());
+        const int s = c->free_slots.take_lowest();
         slot_map_set(c, k, s);
         c->key_of[s] = pack(k);
         c->used[s] = 1;
@@ -775,25 +818,26 @@ int regrid_finish(amr_ctx* c, bool resample_ic, bool* void_step, bool* changed) 
     const auto t1 = std::chrono::steady_clock::now();
     c->regrid_ms[1] = c->regrid_ms[2] = 0.0;
     if (req.empty() && cand.empty()) return AMR_OK;
-    Mesh m2 = c->mesh;
     std::vector<Key> created, deleted;
     {
         Range closure("regrid: closure and coarsening");
-        created = m2.refine(req);
+        created = c->mesh.refine(req);
         std::unordered_set<uint64_t> just;
         for (const auto& k : created) just.insert(pack(k));
-        deleted = m2.coarsen(cand, just);
+        deleted = c->mesh.coarsen(cand, just);
     }
     if (created.empty() && deleted.empty())                // the same candidates give the same answer
         return set_rejected(c, req.empty() ? (int)cand.size() : -1);
-    if ((long long)m2.patches.size() > c->cap)
+    if ((long long)c->mesh.size() > c->cap) {               // taken back
+        for (const auto& k : created) c->mesh.erase(k);
+        for (const auto& k : deleted) c->mesh.insert(k);
         return fail(c, AMR_ERR_POOL, "patch pool capacity exceeded; hierarchy left unchanged");
+    }
     c->ghosts_valid = false;                               // new and removed patches: neighbours' ghosts stale
     if (changed) *changed = true;
     r = set_rejected(c, -1);
     if (r) return r;
     Range tables("regrid: tables and new patches");
-    c->mesh.swap_patches(m2);
     assign_slots(c, created, deleted);
     const auto t2 = std::chrono::steady_clock::now();
     r = rebuild_tables(c, created);
@@ -861,26 +905,23 @@ void* mapped_host(const void* p) {
 
 template <typename T>
 int get_level_impl(amr_ctx* c, int level, int* n_out, int* coords, double* data) {
-    std::vector<int> slots;
-    std::vector<Key> keys;
-    for (size_t i = 0; i < c->canon.size(); ++i)
-        if (c->canon[i].l == level) {
-            keys.push_back(c->canon[i]);
-            slots.push_back(c->canon_slot[i]);
-        }
-    *n_out = (int)keys.size();
+    // the level's patches are one run of the canonical list
+    const int first = c->level_off_h[level], count = c->level_off_h[level + 1] - first;
+    const Key* keys = c->canon.data() + first;
+    const int* slots = c->canon_slot.data() + first;
+    *n_out = count;
     if (coords)
-        for (size_t i = 0; i < keys.size(); ++i) {
+        for (int i = 0; i < count; ++i) {
             const int cc[3] = {keys[i].x, keys[i].y, keys[i].z};
-            for (int d = 0; d < c->dim; ++d) coords[i * c->dim + d] = cc[d];
+            for (int d = 0; d < c->dim; ++d) coords[(size_t)i * c->dim + d] = cc[d];
         }
-    if (data && !slots.empty()) {
+    if (data && count > 0) {
         long long ncell = 1;
         for (int d = 0; d < c->dim; ++d) ncell *= c->N;
         const size_t per = (size_t)c->nv * ncell;
         if (double* dev = static_cast<double*>(mapped_host(data))) {   // straight into the caller's buffer
-            const int n = (int)slots.size();
-            CK(cudaMemcpyAsync(c->slots_d, slots.data(), n * sizeof(int), cudaMemcpyHostToDevice, c->stream),
+            const int n = count;
+            CK(cudaMemcpyAsync(c->slots_d, slots, n * sizeof(int), cudaMemcpyHostToDevice, c->stream),
                "get level");
             CK(Kernels<T>::unpack_interiors(c->grid, St<T>(c, 0), c->slots_d, n, dev, c->stream), "unpack");
             CK(cudaStreamSynchronize(c->stream), "get level");
@@ -890,9 +931,9 @@ int get_level_impl(amr_ctx* c, int level, int* n_out, int* coords, double* data)
             return AMR_OK;
         }
         const size_t chunk = std::max<size_t>(1, c->dense_cap / per);
-        for (size_t b = 0; b < slots.size(); b += chunk) {
-            const int n = (int)std::min(chunk, slots.size() - b);
-            CK(cudaMemcpyAsync(c->slots_d, slots.data() + b, n * sizeof(int), cudaMemcpyHostToDevice, c->stream),
+        for (size_t b = 0; b < (size_t)count; b += chunk) {
+            const int n = (int)std::min(chunk, (size_t)count - b);
+            CK(cudaMemcpyAsync(c->slots_d, slots + b, n * sizeof(int), cudaMemcpyHostToDevice, c->stream),
                "get level");
             CK(Kernels<T>::unpack_interiors(c->grid, St<T>(c, 0), c->slots_d, n, c->dense_d, c->stream), "unpack");
             CK(cudaMemcpyAsync(data + b * per, c->dense_d, n * per * sizeof(double), cudaMemcpyDeviceToHost,
@@ -909,31 +950,36 @@ int get_level_impl(amr_ctx* c, int level, int* n_out, int* coords, double* data)
 
 template <typename T>
 int set_state_impl(amr_ctx* c, int n, const int* levels, const int* coords, const double* data, double t) {
-    Mesh m2(c->dim, c->mesh.base, c->mesh.periodic, c->L - 1);
-    m2.clear();
+    // the new set goes into the context's mesh in place; a set that is refused is
+    // taken out again and the old one put back
+    Mesh& m = c->mesh;
+    const std::vector<uint64_t> old = m.keys;
+    auto refuse = [&](int code, const std::string& why) {
+        m.clear();
+        for (uint64_t v : old) m.insert(unpack(v));
+        return fail(c, code, why);
+    };
+    m.clear();
     std::vector<Key> keys;
+    keys.reserve((size_t)n);
     for (int i = 0; i < n; ++i) {
         Key k{levels[i], coords[i * c->dim], c->dim >= 2 ? coords[i * c->dim + 1] : 0,
               c->dim == 3 ? coords[i * c->dim + 2] : 0};
-        if (k.l < 0 || k.l >= c->L) return fail(c, AMR_ERR_MESH, "level out of range");
+        if (k.l < 0 || k.l >= c->L) return refuse(AMR_ERR_MESH, "level out of range");
         for (int d = 0; d < c->dim; ++d) {                  // before packing: keys hold 20-bit coordinates
             const int x = coords[i * c->dim + d];
-            if (x < 0 || x >= m2.extent(k.l, d)) return fail(c, AMR_ERR_MESH, "patch outside the domain");
+            if (x < 0 || x >= m.extent(k.l, d)) return refuse(AMR_ERR_MESH, "patch outside the domain");
         }
-        if (!m2.insert(k)) return fail(c, AMR_ERR_MESH, "duplicate patch");
+        if (!m.insert(k)) return refuse(AMR_ERR_MESH, "duplicate patch");
         keys.push_back(k);
     }
-    const std::string why = m2.check();
-    if (!why.empty()) return fail(c, AMR_ERR_MESH, why);
-    if ((int)keys.size() > c->cap) return fail(c, AMR_ERR_POOL, "patch pool capacity exceeded");
-    c->mesh.swap_patches(m2);
+    const std::string why = m.check();
+    if (!why.empty()) return refuse(AMR_ERR_MESH, why);
+    if ((int)keys.size() > c->cap) return refuse(AMR_ERR_POOL, "patch pool capacity exceeded");
     slot_map_clear(c);
     c->slot_hi = 0;
-    c->free_slots.clear();
-    for (int s = 0; s < c->cap; ++s) {
-        c->free_slots.insert(s);
-        c->used[s] = 0;
-    }
+    c->free_slots.fill(c->cap);
+    std::fill(c->used.begin(), c->used.end(), 0);
     std::vector<Key> all = c->mesh.canonical();
     assign_slots(c, all, {});
     c->ghosts_valid = false;
@@ -1407,7 +1453,7 @@ int amr_init(amr_ctx** out, const amr_domain_t* dom, double gamma, const int bas
     c->initialising = true;
     c->used.assign(c->cap, 0);
     c->key_of.assign(c->cap, 0);
-    for (int s = 0; s < c->cap; ++s) c->free_slots.insert(s);
+    c->free_slots.fill(c->cap);
     slot_map_clear(c);
     c->slot_hi = 0;
     std::vector<Key> base = c->mesh.canonical();

@@ -19,7 +19,7 @@ Mesh::Mesh(int dim_, const int base_[3], const bool periodic_[3], int max_level_
         o += (long long)extent(l, 0) * extent(l, 1) * extent(l, 2);
     }
     for (int l = max_level + 1; l < 9; ++l) lvl_off[l] = o;
-    if (o <= kDenseMax) present.assign((size_t)o, 0);
+    if (o <= kDenseMax) at.assign((size_t)o, -1);
     // R1: the level-0 Cartesian layout is the permanent scaffold
     for (int z = 0; z < base[2]; ++z)
         for (int y = 0; y < base[1]; ++y)
@@ -69,8 +69,8 @@ std::vector<Key> Mesh::children(const Key& k) const {
 
 std::vector<Key> Mesh::canonical() const {
     std::vector<Key> out;
-    out.reserve(patches.size());
-    if (dense() && (long long)patches.size() * 16 >= positions()) {
+    out.reserve(size());
+    if (dense() && (long long)size() * 16 >= positions()) {
         // the position order is the canonical order
         for (int l = 0; l <= max_level; ++l) {
             const int ex = extent(l, 0), ey = extent(l, 1), ez = extent(l, 2);
@@ -78,11 +78,11 @@ std::vector<Key> Mesh::canonical() const {
             for (int z = 0; z < ez; ++z)
                 for (int y = 0; y < ey; ++y)
                     for (int x = 0; x < ex; ++x, ++p)
-                        if (present[(size_t)p]) out.push_back(Key{l, x, y, z});
+                        if (at[(size_t)p] >= 0) out.push_back(Key{l, x, y, z});
         }
         return out;
     }
-    for (uint64_t v : patches) out.push_back(unpack(v));
+    for (uint64_t v : keys) out.push_back(unpack(v));
     std::sort(out.begin(), out.end(), canon_less);
     return out;
 }
@@ -96,7 +96,9 @@ std::string Mesh::check() const {
                     why << "level-0 patch (" << x << "," << y << "," << z << ") missing (R1)";
                     return why.str();
                 }
-    for (uint64_t v : patches) {
+    const int nz = dim == 3 ? 2 : 1, ny = dim >= 2 ? 2 : 1;
+    const int rz = dim == 3 ? 1 : 0, ry = dim >= 2 ? 1 : 0;
+    for (uint64_t v : keys) {
         const Key k = unpack(v);
         if (k.l < 0 || k.l > max_level) {
             why << "patch beyond the finest level";
@@ -111,20 +113,25 @@ std::string Mesh::check() const {
             why << "patch without parent";
             return why.str();
         }
-        const auto ch = children(k);
         int present = 0;
-        for (const auto& c : ch) present += exists(c);
-        if (present != 0 && present != (int)ch.size()) {
+        for (int sz = 0; sz < nz; ++sz)
+            for (int sy = 0; sy < ny; ++sy)
+                for (int sx = 0; sx < 2; ++sx)
+                    present += exists(Key{k.l + 1, 2 * k.x + sx, dim >= 2 ? 2 * k.y + sy : 0, dim == 3 ? 2 * k.z + sz : 0});
+        if (present != 0 && present != 2 * ny * nz) {
             why << "incomplete sibling group";
             return why.str();
         }
-        if (present) {
-            for (const auto& q : moore(k))
-                if (!exists(q)) {
-                    why << "R2 violated: a refined patch lacks a Moore neighbour";
-                    return why.str();
+        if (!present) continue;
+        for (int oz = -rz; oz <= rz; ++oz)
+            for (int oy = -ry; oy <= ry; ++oy)
+                for (int ox = -1; ox <= 1; ++ox) {
+                    Key q{k.l, k.x + ox, k.y + oy, k.z + oz};
+                    if (wrap(q) && !exists(q)) {
+                        why << "R2 violated: a refined patch lacks a Moore neighbour";
+                        return why.str();
+                    }
                 }
-        }
     }
     return std::string();
 }
@@ -247,10 +254,10 @@ extern "C" int amr_mesh_close(int dim, const int base_patches[3], const int peri
     std::unordered_set<uint64_t> just;
     for (const auto& k : created) just.insert(amr::pack(k));
     const std::vector<Key> deleted = m.coarsen(cand, just);
-    *n_out = (int)m.patches.size();
+    *n_out = (int)m.size();
     if (n_created) *n_created = (int)created.size();
     if (n_deleted) *n_deleted = (int)deleted.size();
-    if ((long long)m.patches.size() > cap_out) return AMR_ERR_POOL;
+    if ((long long)m.size() > cap_out) return AMR_ERR_POOL;
     const std::vector<Key> all = m.canonical();
     for (size_t i = 0; i < all.size(); ++i) {
         out_keys[4 * i + 0] = all[i].l;

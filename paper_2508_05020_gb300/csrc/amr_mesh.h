@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <algorithm>
 #include <string>
+#include <unordered_map>
 #include <unordered_set>
 #include <vector>
 
@@ -44,17 +45,19 @@ public:
     int dim = 1, max_level = 0;
     int base[3] = {1, 1, 1};
     bool periodic[3] = {false, false, false};
-    // the patch set; read freely, change only through insert / erase / clear /
-    // swap_patches, which keep the position index below in step
-    std::unordered_set<uint64_t> patches;
+    // The patch set: the packed keys in no particular order, and the index of
+    // every patch among them. Change it only through insert / erase / clear.
+    std::vector<uint64_t> keys;
     // Dense position index of every patch position a level can hold: level
-    // by level, then lexicographic (z, y, x), i.e. the canonical order. Used
-    // (present non-empty) when all positions fit in kDenseMax; a membership
-    // test is then one array read.
+    // by level, then lexicographic (z, y, x), i.e. the canonical order; holds
+    // the index in `keys`, -1 if there is no patch. Used (at non-empty) when all
+    // positions fit in kDenseMax; a membership test is then one array read.
     static constexpr long long kDenseMax = 1ll << 26;
     long long lvl_off[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    std::vector<uint8_t> present;
+    std::vector<int> at;
+    std::unordered_map<uint64_t, int> index;        // the same without a dense index
 
+    size_t size() const { return keys.size(); }
     int extent(int level, int d) const { return d < dim ? base[d] << level : 1; }
     // position of k in the dense index, -1 outside the levels or the domain
     long long pos(const Key& k) const {
@@ -64,33 +67,48 @@ public:
         return lvl_off[k.l] + ((long long)k.z * ey + k.y) * ex + k.x;
     }
     long long positions() const { return lvl_off[max_level + 1]; }
-    bool dense() const { return !present.empty(); }
+    bool dense() const { return !at.empty(); }
     bool exists(const Key& k) const {
         if (dense()) {
             const long long p = pos(k);
-            return p >= 0 && present[(size_t)p];
+            return p >= 0 && at[(size_t)p] >= 0;
         }
-        return patches.count(pack(k)) != 0;
+        return index.count(pack(k)) != 0;
     }
     // false if k is present already (or, with the dense index, outside it)
     bool insert(const Key& k) {
-        const long long p = dense() ? pos(k) : 0;
-        if (p < 0 || !patches.insert(pack(k)).second) return false;
-        if (dense()) present[(size_t)p] = 1;
+        const uint64_t v = pack(k);
+        if (dense()) {
+            const long long p = pos(k);
+            if (p < 0 || at[(size_t)p] >= 0) return false;
+            at[(size_t)p] = (int)keys.size();
+        } else if (!index.emplace(v, (int)keys.size()).second) {
+            return false;
+        }
+        keys.push_back(v);
         return true;
     }
     bool erase(const Key& k) {
-        if (!patches.erase(pack(k))) return false;
-        if (dense()) present[(size_t)pos(k)] = 0;
+        if (!exists(k)) return false;
+        int* mine = dense() ? &at[(size_t)pos(k)] : &index.find(pack(k))->second;
+        const int i = *mine;
+        const uint64_t last = keys.back();           // takes the place of k in the list
+        keys[(size_t)i] = last;
+        keys.pop_back();
+        if (dense()) {
+            at[(size_t)pos(unpack(last))] = i;
+            *mine = -1;
+        } else {
+            index.find(last)->second = i;
+            index.erase(pack(k));
+        }
         return true;
     }
     void clear() {
-        patches.clear();
-        std::fill(present.begin(), present.end(), 0);
-    }
-    void swap_patches(Mesh& o) {
-        patches.swap(o.patches);
-        present.swap(o.present);
+        if (dense())
+            for (uint64_t v : keys) at[(size_t)pos(unpack(v))] = -1;
+        index.clear();
+        keys.clear();
     }
     // wrap coordinates across periodic dimensions; false if outside the domain
     bool wrap(Key& k) const;
