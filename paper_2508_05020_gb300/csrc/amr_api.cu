@@ -100,8 +100,9 @@ struct amr_ctx {
     int* meta_h = nullptr;                     // pinned mirror
     size_t meta_ints = 0;
     int* anyflag = nullptr;
-    int* req_d = nullptr;                      // [3 + 3 cap]: counts, refine, coarsen, rejected candidates
-    int* rej_d = nullptr;                      // req_d + 2 + 2 cap: [count or -1, slots] the host could not coarsen
+    // [REQ_HEAD + 1 + 3 cap]: counts, error bits and cancel word, refine, coarsen, rejected candidates
+    int* req_d = nullptr;
+    int* rej_d = nullptr;                      // after the lists: [count or -1, slots] the host could not coarsen
     int* req_h = nullptr;
     double* cons_partial = nullptr;
     double* cons_d = nullptr;
@@ -733,17 +734,19 @@ int regrid_enqueue(amr_ctx* c) {
            "flag");
     }
     CK(mark(c->ev_rg[2]), "event");
-    CK(launch_requests(c->grid, c->anyflag, c->rej_d, c->req_d + 2, c->req_d + 2 + c->cap, c->req_d, c->stream),
+    CK(launch_requests(c->grid, c->anyflag, c->rej_d, c->req_d + REQ_HEAD, c->req_d + REQ_HEAD + c->cap, c->req_d,
+                       c->stream),
        "requests");
     c->kernels += 2;
-    // counts and the first REQ_READ entries of both lists, and the time record, in one read-back
+    // the head and the first REQ_READ entries of both lists (one copy where they are whole)
     const int head = std::min(c->cap, REQ_READ);
-    CK(cudaMemcpyAsync(c->req_h, c->req_d, (2 + (size_t)head) * sizeof(int), cudaMemcpyDeviceToHost, c->stream),
+    const size_t lists = head == c->cap ? 2 * (size_t)c->cap : (size_t)head;
+    CK(cudaMemcpyAsync(c->req_h, c->req_d, (REQ_HEAD + lists) * sizeof(int), cudaMemcpyDeviceToHost, c->stream),
        "read requests");
-    CK(cudaMemcpyAsync(c->req_h + 2 + c->cap, c->req_d + 2 + c->cap, (size_t)head * sizeof(int),
-                       cudaMemcpyDeviceToHost, c->stream),
-       "read requests");
-    CK(cudaMemcpyAsync(c->time_h, c->time_d, sizeof(DevTime), cudaMemcpyDeviceToHost, c->stream), "read time");
+    if (head < c->cap)
+        CK(cudaMemcpyAsync(c->req_h + REQ_HEAD + c->cap, c->req_d + REQ_HEAD + c->cap, (size_t)head * sizeof(int),
+                           cudaMemcpyDeviceToHost, c->stream),
+           "read requests");
     CK(cudaEventRecord(c->ev_req, c->stream), "read requests");
     c->ghosts_valid = true;                                // filled at the current time for the flags
     return AMR_OK;
@@ -754,19 +757,21 @@ int regrid_enqueue(amr_ctx* c) {
 // compaction set DevTime::cancel, so a step issued after regrid_enqueue is void.
 int read_requests(amr_ctx* c, std::vector<Key>& req, std::vector<Key>& cand, bool* void_step = nullptr) {
     CK(cudaEventSynchronize(c->ev_req), "read requests");
+    c->time_h->err = c->req_h[2];
+    c->time_h->cancel = c->req_h[3];
     if (void_step) *void_step = c->time_h->cancel != 0;
     const int nr = c->req_h[0], nc = c->req_h[1];
     const int head = std::min(c->cap, REQ_READ);
-    c->d2h += (long long)(2 + 2 * head) * sizeof(int) + sizeof(DevTime);
+    c->d2h += (long long)(REQ_HEAD + 2 * head) * sizeof(int);
     if (nr | nc) {
         CK(cudaMemsetAsync(&c->time_d->cancel, 0, sizeof(int), c->stream), "clear cancel");
         if (nr > head || nc > head) {                      // long lists: the rest in a second read-back
             if (nr > head)
-                CK(cudaMemcpyAsync(c->req_h + 2 + head, c->req_d + 2 + head, (size_t)(nr - head) * sizeof(int),
+                CK(cudaMemcpyAsync(c->req_h + REQ_HEAD + head, c->req_d + REQ_HEAD + head, (size_t)(nr - head) * sizeof(int),
                                    cudaMemcpyDeviceToHost, c->stream),
                    "read requests");
             if (nc > head)
-                CK(cudaMemcpyAsync(c->req_h + 2 + c->cap + head, c->req_d + 2 + c->cap + head,
+                CK(cudaMemcpyAsync(c->req_h + REQ_HEAD + c->cap + head, c->req_d + REQ_HEAD + c->cap + head,
                                    (size_t)(nc - head) * sizeof(int), cudaMemcpyDeviceToHost, c->stream),
                    "read requests");
             CK(cudaStreamSynchronize(c->stream), "read requests");
@@ -777,8 +782,8 @@ int read_requests(amr_ctx* c, std::vector<Key>& req, std::vector<Key>& cand, boo
     if (r) return r;
     req.clear();
     cand.clear();
-    for (int i = 0; i < nr; ++i) req.push_back(unpack(c->key_of[c->req_h[2 + i]]));
-    for (int i = 0; i < nc; ++i) cand.push_back(unpack(c->key_of[c->req_h[2 + c->cap + i]]));
+    for (int i = 0; i < nr; ++i) req.push_back(unpack(c->key_of[c->req_h[REQ_HEAD + i]]));
+    for (int i = 0; i < nc; ++i) cand.push_back(unpack(c->key_of[c->req_h[REQ_HEAD + c->cap + i]]));
     c->regrid_ms[0] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - c->rg_t0).count();
     c->regrid_timed = c->timing;
     return AMR_OK;
@@ -795,10 +800,10 @@ int compute_requests(amr_ctx* c, std::vector<Key>& req, std::vector<Key>& cand) 
 // The device copy of the coarsening candidates the host found it could not
 // coarsen (n >= 0), or none (n = -1), for the request compaction's test.
 int set_rejected(amr_ctx* c, int n) {
-    int* stage = c->req_h + 2 + 2 * (size_t)c->cap;      // pinned staging word
+    int* stage = c->req_h + REQ_HEAD + 2 * (size_t)c->cap;      // pinned staging word
     *stage = n;
     if (n > 0)
-        CK(cudaMemcpyAsync(c->rej_d + 1, c->req_d + 2 + c->cap, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice,
+        CK(cudaMemcpyAsync(c->rej_d + 1, c->req_d + REQ_HEAD + c->cap, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice,
                            c->stream),
            "rejected");
     CK(cudaMemcpyAsync(c->rej_d, stage, sizeof(int), cudaMemcpyHostToDevice, c->stream), "rejected");
@@ -1352,7 +1357,7 @@ int amr_init(amr_ctx** out, const amr_domain_t* dom, double gamma, const int bas
     c->meta_ints = ml.total;
     c->meta_d = (int*)dalloc(c, ml.total * sizeof(int));
     c->anyflag = (int*)dalloc(c, (c->cap + 32) * sizeof(int));     // flags + the learned flagger's work counter
-    c->req_d = (int*)dalloc(c, (3 + 3 * (size_t)c->cap) * sizeof(int));
+    c->req_d = (int*)dalloc(c, (REQ_HEAD + 1 + 3 * (size_t)c->cap) * sizeof(int));
     c->cons_partial = (double*)dalloc(c, (size_t)c->cap * c->nv * sizeof(double));
     c->cons_d = (double*)dalloc(c, 8 * sizeof(double));
     c->dense_cap = std::max<size_t>((size_t)g.patch_elems * 64, (size_t)1 << 22);
@@ -1366,11 +1371,11 @@ int amr_init(amr_ctx** out, const amr_domain_t* dom, double gamma, const int bas
         !c->slots_d || !c->time_d)
         return fail(c, AMR_ERR_CUDA, "device allocation failed");
     if (cudaMallocHost((void**)&c->meta_h, ml.total * sizeof(int)) != cudaSuccess ||
-        cudaMallocHost((void**)&c->req_h, (3 + 2 * (size_t)c->cap) * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost((void**)&c->req_h, (REQ_HEAD + 1 + 2 * (size_t)c->cap) * sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void**)&c->time_h, sizeof(DevTime)) != cudaSuccess)
         return fail(c, AMR_ERR_CUDA, "pinned host allocation failed");
     CK(cudaEventCreateWithFlags(&c->ev_req, cudaEventDisableTiming), "event");
-    c->rej_d = c->req_d + 2 + 2 * (size_t)c->cap;
+    c->rej_d = c->req_d + REQ_HEAD + 2 * (size_t)c->cap;
     CK(cudaMemsetAsync(c->rej_d, 0xFF, sizeof(int), c->stream), "clear rejected");   // -1: none
     for (int i = 0; i < 3; ++i) CK(cudaMemsetAsync(c->U[i], 0, state_bytes, c->stream), "clear pool");
     CK(cudaMemsetAsync(c->faces, 0, face_bytes, c->stream), "clear faces");

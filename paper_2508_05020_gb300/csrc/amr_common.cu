@@ -115,6 +115,8 @@ __global__ void __launch_bounds__(1024) k_requests(Grid g, const int* anyflag, c
     if (threadIdx.x == 0) {
         out_counts[0] = nr;
         out_counts[1] = nc;
+        out_counts[2] = g.time->err;
+        out_counts[3] = cancel;
         g.time->cancel = cancel;
     }
 }

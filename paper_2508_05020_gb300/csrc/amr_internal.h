@@ -183,6 +183,10 @@ struct Kernels {
                                unsigned char* labels, int max_n, cudaStream_t s);
 };
 
+// words before the request lists: refinement requests, coarsening candidates,
+// error bits and cancel word of the time record
+constexpr int REQ_HEAD = 4;
+
 // dt finalisation and request compaction (precision-independent, amr_common.cu)
 cudaError_t launch_finalize_dt(const Grid& g, cudaStream_t s);
 cudaError_t launch_set_dt(DevTime* t, double dt, cudaStream_t s);

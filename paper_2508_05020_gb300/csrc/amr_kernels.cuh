@@ -658,6 +658,18 @@ __device__ __forceinline__ void hybrid_flux(const T (&p)[6], const T (&un)[6], c
     }
 }
 
+// The words a step's kernel starts from, loaded together before the test of any
+// of them: a small launch is a chain of dependent loads, and each link it
+// saves is 0.3 us of a launch of three.
+struct LaunchWords {
+    int cancel;                                          // a void step (see DevTime::cancel): return
+    int n_all, n_leaf, n_reflux;
+    double t, dt;
+    __device__ __forceinline__ explicit LaunchWords(const Grid& g)
+        : cancel(g.time->cancel), n_all(g.counts[0]), n_leaf(g.counts[1]), n_reflux(g.counts[2]), t(g.time->t),
+          dt(g.time->dt) {}
+};
+
 // Metadata of one patch staged in shared memory by the CTA that serves it:
 // level, coordinates, its 27-entry neighbour table and its parent's.
 struct PatchMeta {
@@ -977,15 +989,15 @@ __device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* 
 // shared-memory copy; warps never wait for one another.
 // ---------------------------------------------------------------------------
 template <typename T, int D, int N, bool STAGE>
-__device__ __forceinline__ void ghost_items(const Grid& g, T* U, double tfrac, int one_slot, double4 pre, double4 post,
-                                            int chunk, int n_cells, int warp, int nw, PatchMeta& m) {
+__device__ __forceinline__ void ghost_items(const Grid& g, T* U, double t, int n_all, int one_slot, double4 pre,
+                                            double4 post, int chunk, int n_cells, int warp, int nw, PatchMeta& m) {
     constexpr bool stage_only = STAGE;                  // compiled apart: the full fill keeps its registers
     constexpr int NV = D + 2;
     const int lane = threadIdx.x & 31;
-    const int npatch = one_slot >= 0 ? 1 : g.counts[0];
+    const int npatch = one_slot >= 0 ? 1 : n_all;
     const double pr[4] = {pre.x, pre.y, pre.z, pre.w};
     const double po[4] = {post.x, post.y, post.z, post.w};
-    const BcState bc{g.time->t + tfrac * g.time->dt, pr, po};
+    const BcState bc{t, pr, po};
     // a stage walks the 2d face boxes of a patch (G N^(d-1) table entries
     // each) and skips a box whole when a same-level neighbour lies across it
     constexpr int BOX = G * (D == 1 ? 1 : (D == 2 ? N : N * N));
@@ -1085,10 +1097,11 @@ template <typename T, int D, int N, bool STAGE>
 __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(Grid g, T* U, double tfrac, int one_slot,
                                                double4 pre, double4 post, int chunk, int n_cells) {
     __shared__ PatchMeta metas[256 / 32];
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
+    const LaunchWords w(g);
+    if (w.cancel) return;
     const int warp = threadIdx.x >> 5;
-    ghost_items<T, D, N, STAGE>(g, U, tfrac, one_slot, pre, post, chunk, n_cells, blockIdx.x * (256 / 32) + warp,
-                                gridDim.x * (256 / 32), metas[warp]);
+    ghost_items<T, D, N, STAGE>(g, U, w.t + tfrac * w.dt, w.n_all, one_slot, pre, post, chunk, n_cells,
+                                blockIdx.x * (256 / 32) + warp, gridDim.x * (256 / 32), metas[warp]);
 }
 
 // Restriction mean of the 2^d children of a covered coarse cell, given in
@@ -1333,9 +1346,13 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
     constexpr int NT = D - 1;
     constexpr int CPT = (C::CELLS + NTH - 1) / NTH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
+    const LaunchWords words(g);
+    // the slot of the first item too (a list entry of the pool in any case)
+    const int first = blockIdx.x / C::NCH;
+    int next_slot = one_slot >= 0 ? one_slot : g.leaf_list[first < g.cap ? first : 0];
+    if (words.cancel) return;
     // the step's last stage moves the time on: nothing after it in the step reads it
-    if ((flags & RHS_ADVANCE) && blockIdx.x == 0 && threadIdx.x == 0) g.time->t = g.time->t + g.time->dt;
+    if ((flags & RHS_ADVANCE) && blockIdx.x == 0 && threadIdx.x == 0) g.time->t = words.t + words.dt;
     unsigned char* sbase = smem_raw;
     if constexpr (TMA)                                   // tensor-copy destinations: 128-byte aligned
         sbase += (128u - (rhs_smem_addr(smem_raw) & 127u)) & 127u;
@@ -1354,22 +1371,21 @@ __global__ void __launch_bounds__(NTH, MINB) k_rhs(Grid g, const T* __restrict__
     }
     const T gamma = T(g.gamma);
     const T gm1 = T(g.gamma) - T(1);
-    const double dtd = g.time->dt;
-    const T dt = T(dtd);
+    const T dt = T(words.dt);
     const T ra = stage == 0 ? T(0) : (stage == 1 ? T(0.75) : T(1.0 / 3.0));
     const T rb = stage == 0 ? T(1) : (stage == 1 ? T(0.25) : T(2.0 / 3.0));
     // leaves only: a patch with children is covered by them, and the
     // restriction after the stage overwrites its whole interior
-    const int npatch = one_slot >= 0 ? 1 : g.counts[1];
+    const int npatch = one_slot >= 0 ? 1 : words.n_leaf;
     const int n_items = npatch * C::NCH;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const int pi = item / C::NCH;
-        const int ch0 = item - pi * C::NCH;
+        const int ch0 = item % C::NCH;
         const int z0 = ch0 / C::NCHY * DZ;               // first interior plane (3D) and row of the chunk
         const int y0 = D >= 2 ? ch0 % C::NCHY * DY : 0;
-        const int slot = one_slot >= 0 ? one_slot : g.leaf_list[pi];
+        const int slot = next_slot;
         const int lev = g.level[slot];
         const int pf = g.pflag[slot];
+        if (item + gridDim.x < n_items && one_slot < 0) next_slot = g.leaf_list[(item + gridDim.x) / C::NCH];
         const bool fuse = (flags & RHS_RESTRICT) && lev == g.L - 1 && lev >= 1;
         // 1. stage the chunk and its halo as primitives, loading 16-byte vectors
         //    along x (slot rows are 16-byte aligned)
@@ -1890,9 +1906,10 @@ __device__ __forceinline__ T stage_b(int stage) {
 template <typename T, int D, int N>
 __global__ void __launch_bounds__(256) k_reflux(Grid g, T* Uout, const T* __restrict__ faces, int stage,
                                                 int one_item) {
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
-    const T dt = T(g.time->dt);
-    const int n = one_item >= 0 ? one_item + 1 : g.counts[2];
+    const LaunchWords w(g);
+    if (w.cancel) return;
+    const T dt = T(w.dt);
+    const int n = one_item >= 0 ? one_item + 1 : w.n_reflux;
     for (int e = one_item >= 0 ? one_item : blockIdx.x; e < n; e += gridDim.x)
         reflux_patch<T, D, N>(g, Uout, faces, stage_b<T>(stage), dt, e);
 }
@@ -1903,7 +1920,7 @@ __global__ void __launch_bounds__(256) k_reflux(Grid g, T* Uout, const T* __rest
 // summed in FP64 (FP32 fields: an error-free FP32 pair sum, rounded once)
 // ---------------------------------------------------------------------------
 template <typename T, int D, int N>
-__device__ __forceinline__ void restrict_items(const Grid& g, T* U, int level, int one_slot, long long thread,
+__device__ __forceinline__ void restrict_items(const Grid& g, T* U, int lo, int hi, int one_slot, long long thread,
                                                long long nthreads) {
     // thread <-> CP coarse cells adjacent in x (FP32: 2, FP64: 1), whose
     // children of each (y, z) offset are VE consecutive fine cells of a row:
@@ -1915,7 +1932,6 @@ __device__ __forceinline__ void restrict_items(const Grid& g, T* U, int level, i
     constexpr int HC = (D == 1 ? H : (D == 2 ? H * H : H * H * H)) / CP;
     constexpr int NYZ = 1 << (D - 1);                    // child (y, z) offsets
     constexpr int NCH = 1 << D;
-    const int lo = g.level_off[level], hi = g.level_off[level + 1];
     const int npatch = one_slot >= 0 ? 1 : hi - lo;
     const long long total = (long long)npatch * HC;
     for (long long it = thread; it < total; it += nthreads) {
@@ -1957,8 +1973,9 @@ __device__ __forceinline__ void restrict_items(const Grid& g, T* U, int level, i
 
 template <typename T, int D, int N>
 __global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int one_slot) {
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
-    restrict_items<T, D, N>(g, U, level, one_slot, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
+    const int cancel = g.time->cancel, lo = g.level_off[level], hi = g.level_off[level + 1];
+    if (cancel) return;                                  // a void step (see DevTime::cancel)
+    restrict_items<T, D, N>(g, U, lo, hi, one_slot, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
 }
 
 // ---------------------------------------------------------------------------
@@ -1983,18 +2000,20 @@ __global__ void __cluster_dims__(AFTER_CTAS, 1, 1) __launch_bounds__(256)
     k_after(Grid g, T* U, const T* __restrict__ faces, int stage, int next, double tfrac, double4 pre, double4 post,
             int chunk, int n_cells) {
     __shared__ PatchMeta metas[256 / 32];
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
-    const T dt = T(g.time->dt);
-    for (int e = blockIdx.x; e < g.counts[2]; e += AFTER_CTAS)
+    const LaunchWords w(g);
+    if (w.cancel) return;
+    const T dt = T(w.dt);
+    for (int e = blockIdx.x; e < w.n_reflux; e += AFTER_CTAS)
         reflux_patch<T, D, N>(g, U, faces, stage_b<T>(stage), dt, e);
     for (int l = g.L - 2; l >= 1; --l) {                 // level L - 1: fused into the RHS
         cluster_barrier();
-        restrict_items<T, D, N>(g, U, l, -1, blockIdx.x * 256 + threadIdx.x, AFTER_CTAS * 256);
+        restrict_items<T, D, N>(g, U, g.level_off[l], g.level_off[l + 1], -1, blockIdx.x * 256 + threadIdx.x,
+                                AFTER_CTAS * 256);
     }
     if (!next) return;
     cluster_barrier();
     const int warp = threadIdx.x >> 5;
-    ghost_items<T, D, N, true>(g, U, tfrac, -1, pre, post, chunk, n_cells, blockIdx.x * (256 / 32) + warp,
+    ghost_items<T, D, N, true>(g, U, w.t + tfrac * w.dt, w.n_all, -1, pre, post, chunk, n_cells, blockIdx.x * (256 / 32) + warp,
                                AFTER_CTAS * (256 / 32), metas[warp]);
 }
 
@@ -2014,8 +2033,9 @@ __global__ void __launch_bounds__(256) k_cfl(Grid g, const T* U, int one_slot, i
     constexpr int NV = D + 2;
     constexpr int VE = Vec16<T>::VE;
     constexpr int NC = (D == 1 ? N : (D == 2 ? N * N : N * N * N)) / VE;
-    if (g.time->cancel) return;                          // a void step (see DevTime::cancel)
-    const int npatch = one_slot >= 0 ? 1 : g.counts[1];
+    const LaunchWords w(g);
+    if (w.cancel) return;
+    const int npatch = one_slot >= 0 ? 1 : w.n_leaf;
     const long long total = (long long)npatch * NC;
     const T gamma = T(g.gamma);
     const T gm1 = T(g.gamma) - T(1);
@@ -2181,7 +2201,10 @@ __global__ void __launch_bounds__(256) k_flag_plain(Grid g, const T* U, int* any
             any = any || f;
         }
         const int res = __syncthreads_or(any);
-        if (threadIdx.x == 0 && res) atomicOr(&anyflag[slot], 3);   // refine and keep
+        if (threadIdx.x == 0) {                          // refine and keep
+            if constexpr (F::NSLAB == 1) anyflag[slot] = res ? 3 : 0;
+            else if (res) atomicOr(&anyflag[slot], 3);
+        }
     }
 }
 
