@@ -139,7 +139,8 @@ constexpr int ROWS_NTH = 512;
 constexpr int ROWS_CL = 4;                  // blocks of a cluster, whose parts are added in shared memory
 constexpr int ROWS_MAXCL = 32;              // clusters of a launch
 constexpr int W1_CT = 16;                   // columns of X of a k_w1grad block
-constexpr int W1_RC = 64;                   // rows staged at a time
+constexpr int W1_NTH = 512, W1_G = W1_NTH / 64;   // threads of a k_w1grad block, its row groups
+constexpr int W1_RC = 128;                  // rows staged at a time
 constexpr int W1_PARTS = 160000;            // floats of the split dW1 (4 x 64 x 625)
 
 // row splits of k_w1grad: about one block per SM over the column tiles, as far
@@ -213,6 +214,7 @@ __global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
 #pragma unroll
     for (int i = 0; i < H * H / ROWS_NTH; ++i) aw2[i] = 0.f;
     const long tiles = (n + R - 1) / R;
+    float w2r[H * H / ROWS_NTH];                           // W2 on its way while layer 1 runs
     for (long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const long r0 = tile * R;
         const int nr = (int)(n - r0 < R ? n - r0 : R);
@@ -225,21 +227,35 @@ __global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
             float acc[OW * R];
 #pragma unroll
             for (int i = 0; i < OW * R; ++i) acc[i] = 0.f;
-#pragma unroll 4
-            for (int ks = 0; ks < KS; ++ks) {
+            // W1 is fetched PF lane steps ahead of its use
+            constexpr int PF = KS < 4 ? KS : 4;
+            float wv[PF][OW];
+            auto fetch = [&](int ks, float (&o)[OW]) {
                 const int k = ks * 32 + lane;
-                const int kk = k < K ? k : K - 1;
-                float wv[OW];
 #pragma unroll
-                for (int j = 0; j < OW; ++j) {
-                    const float x = W1[(warp * OW + j) * K + kk];
-                    wv[j] = k < K ? x : 0.f;
-                }
+                for (int j = 0; j < OW; ++j) o[j] = k < K ? W1[(warp * OW + j) * K + k] : 0.f;
+            };
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float x = Xs[r * K + kk];
+            for (int b = 0; b < PF; ++b) fetch(b, wv[b]);
 #pragma unroll
-                    for (int j = 0; j < OW; ++j) acc[j * R + r] = fmaf(x, wv[j], acc[j * R + r]);
+            for (int i = 0; i < H * H / ROWS_NTH; ++i) w2r[i] = W2[t + i * ROWS_NTH];
+#pragma unroll 1
+            for (int k0 = 0; k0 < KS; k0 += PF) {
+#pragma unroll
+                for (int b = 0; b < PF; ++b) {
+                    const int ks = k0 + b, k = ks * 32 + lane;
+                    if (KS % PF != 0 && ks >= KS) break;
+                    const int kk = k < K ? k : K - 1;
+                    float wk[OW];
+#pragma unroll
+                    for (int j = 0; j < OW; ++j) wk[j] = wv[b][j];
+                    if (ks + PF < KS) fetch(ks + PF, wv[b]);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float x = Xs[r * K + kk];
+#pragma unroll
+                        for (int j = 0; j < OW; ++j) acc[j * R + r] = fmaf(x, wk[j], acc[j * R + r]);
+                    }
                 }
             }
             const int base = lane_sums<OW * R>(acc);
@@ -251,7 +267,11 @@ __global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
             }
         }
         __syncthreads();                                   // the rows of X are read; H1 is written
-        for (int i = t; i < H * H; i += ROWS_NTH) W2s[(i >> 6) * P2 + (i & (H - 1))] = W2[i];
+#pragma unroll
+        for (int i = 0; i < H * H / ROWS_NTH; ++i) {
+            const int e = t + i * ROWS_NTH;
+            W2s[(e >> 6) * P2 + (e & (H - 1))] = w2r[i];
+        }
         __syncthreads();
         for (int r = rg; r < R; r += ROWS_NTH / H) {
             float acc = b2[o];
@@ -327,18 +347,19 @@ __global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
     cl.sync();                                             // a block's sums stay until its peers have read them
 }
 
-// dW1 of W1_CT columns over one split of the rows: rows are staged 64 at a time
+// dW1 of W1_CT columns over one split of the rows: rows are staged 128 at a time
 // (the next ones on their way in registers), a thread owns 8 outputs x 2
-// columns and every fourth row, so that 16 FMAs share three shared-memory
-// loads; the four row groups are added in order at the end. FMA issue bound.
+// columns and every eighth row, so that 16 FMAs share three shared-memory
+// loads; the eight row groups are added in order at the end. Bound by the
+// latency of those loads: 16 warps per SM, as 8 left the scheduler idle in 60 % of the cycles.
 template <int D>
-__global__ void __launch_bounds__(256) k_w1grad(const float* __restrict__ dH1, const float* __restrict__ X,
+__global__ void __launch_bounds__(W1_NTH) k_w1grad(const float* __restrict__ dH1, const float* __restrict__ X,
                                                 const int* __restrict__ idx, long n, float* __restrict__ part) {
     constexpr int K = mlp_kin(D), H = MLP_H, CT = W1_CT, RC = W1_RC;
-    constexpr int ND = RC * H / 4 / 256, NX = RC * CT / 256;
+    constexpr int NTH = W1_NTH, ND = RC * H / 4 / NTH, NX = RC * CT / NTH;
     __shared__ __align__(16) float ds[RC * H];
     __shared__ __align__(16) float xs[RC * CT];
-    static_assert(4 * H * CT <= RC * H, "the row groups' sums fit the staged rows");
+    static_assert(W1_G * H * CT <= RC * H, "the row groups' sums fit the staged rows");
     const int t = threadIdx.x, k0 = blockIdx.x * CT;
     const long per = (n + gridDim.y - 1) / gridDim.y;
     const long lo = blockIdx.y * per, hi = lo + per < n ? lo + per : n;
@@ -347,13 +368,13 @@ __global__ void __launch_bounds__(256) k_w1grad(const float* __restrict__ dH1, c
     auto fetch = [&](long b) {
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
-            const int e = t + i * 256;
+            const int e = t + i * NTH;
             const long r = b + (e >> 4);
             rd[i] = r < hi ? *reinterpret_cast<const float4*>(dH1 + r * H + (e & 15) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int i = 0; i < NX; ++i) {
-            const int e = t + i * 256, k = k0 + (e & (CT - 1));
+            const int e = t + i * NTH, k = k0 + (e & (CT - 1));
             const long r = b + e / CT;
             rx[i] = (r < hi && k < K) ? X[(long)(idx ? idx[r] : r) * K + k] : 0.f;
         }
@@ -365,13 +386,14 @@ __global__ void __launch_bounds__(256) k_w1grad(const float* __restrict__ dH1, c
     fetch(lo);
     for (long b = lo; b < hi; b += RC) {
 #pragma unroll
-        for (int i = 0; i < ND; ++i) reinterpret_cast<float4*>(ds)[t + i * 256] = rd[i];
+        for (int i = 0; i < ND; ++i) reinterpret_cast<float4*>(ds)[t + i * NTH] = rd[i];
 #pragma unroll
-        for (int i = 0; i < NX; ++i) xs[t + i * 256] = rx[i];
+        for (int i = 0; i < NX; ++i) xs[t + i * NTH] = rx[i];
         __syncthreads();
         if (b + RC < hi) fetch(b + RC);
+        const int rows = hi - b < RC ? (int)(hi - b) : RC;
 #pragma unroll 4
-        for (int r = g; r < RC; r += 4) {
+        for (int r = g; r < rows; r += W1_G) {
             const float4 a = *reinterpret_cast<const float4*>(ds + r * H + og * 8);
             const float4 c = *reinterpret_cast<const float4*>(ds + r * H + og * 8 + 4);
             const float2 x = *reinterpret_cast<const float2*>(xs + r * CT + kg * 2);
@@ -390,10 +412,12 @@ __global__ void __launch_bounds__(256) k_w1grad(const float* __restrict__ dH1, c
         ds[(g * H + og * 8 + i) * CT + kg * 2 + 1] = acc[i][1];
     }
     __syncthreads();
-    for (int e = t; e < H * CT; e += 256) {
+    for (int e = t; e < H * CT; e += NTH) {
         const int k = k0 + (e & (CT - 1));
-        if (k < K)
-            part[((long)blockIdx.y * H + e / CT) * K + k] = ((ds[e] + ds[H * CT + e]) + ds[2 * H * CT + e]) + ds[3 * H * CT + e];
+        float sum = ds[e];
+#pragma unroll
+        for (int q = 1; q < W1_G; ++q) sum += ds[q * H * CT + e];
+        if (k < K) part[((long)blockIdx.y * H + e / CT) * K + k] = sum;
     }
 }
 
@@ -490,8 +514,8 @@ int fwd_bwd_d(const float* X, const int* idx, const float* y, long n, float pw, 
     if (R == 4) k_rows<D, 4><<<grid, ROWS_NTH, 0, s>>>(X, idx, y, n, pw, w, sc.dH1, sc.small);
     else if (R == 8) k_rows<D, 8><<<grid, ROWS_NTH, 0, s>>>(X, idx, y, n, pw, w, sc.dH1, sc.small);
     else k_rows<D, 16><<<grid, ROWS_NTH, 0, s>>>(X, idx, y, n, pw, w, sc.dH1, sc.small);
-    const int splits = (int)std::min<long>(w1_splits(K), (n + W1_RC - 1) / W1_RC);
-    k_w1grad<D><<<dim3(w1_tiles(K), splits), 256, 0, s>>>(sc.dH1, X, idx, n, sc.w1);
+    const int splits = (int)std::min<long>(w1_splits(K), (n + 63) / 64);
+    k_w1grad<D><<<dim3(w1_tiles(K), splits), W1_NTH, 0, s>>>(sc.dH1, X, idx, n, sc.w1);
     k_gradsum<<<(MLP_H * K + SMALL_L + 255) / 256, 256, 0, s>>>(K, sc.w1, splits, sc.small, ncl, g, loss, loss_scale,
                                                                 add, adam);
     return cudaGetLastError() == cudaSuccess ? AMR_OK : AMR_ERR_CUDA;
