@@ -18,15 +18,17 @@ namespace amr {
 // arithmetic helpers: FP64 uses IEEE division and square root; FP32 uses the
 // fast approximate forms (the FP32 path is compared by tolerance, not bits)
 // ---------------------------------------------------------------------------
-// half(a, b): a / 2 + b with a / 2 exact, so the fused form rounds as the two operations do
+// half(a, b), quarter(a, b): a / 2 + b, a / 4 + b; the products are exact, so the fused forms round as the two operations do
 template <typename T> struct Num;
 template <> struct Num<double> {
     __device__ __forceinline__ static double half(double a, double b) { return __fma_rn(0.5, a, b); }
+    __device__ __forceinline__ static double quarter(double a, double b) { return __fma_rn(0.25, a, b); }
     __device__ __forceinline__ static double div(double a, double b) { return a / b; }
     __device__ __forceinline__ static double sqr(double a) { return sqrt(a); }
 };
 template <> struct Num<float> {
     __device__ __forceinline__ static float half(float a, float b) { return 0.5f * a + b; }
+    __device__ __forceinline__ static float quarter(float a, float b) { return 0.25f * a + b; }
     __device__ __forceinline__ static float div(float a, float b) { return __fdividef(a, b); }
     __device__ __forceinline__ static float sqr(float a) { return sqrtf(a); }
 };
@@ -863,16 +865,37 @@ __device__ __forceinline__ void prolong_child(const T (&UC)[D + 2], const T (&sl
     for (int d = 0; d < D; ++d) {
         const bool up = (ch >> d) & 1;
 #pragma unroll
-        for (int k = 0; k < D + 2; ++k) v[k] = up ? v[k] + T(0.25) * slope[d][k] : v[k] - T(0.25) * slope[d][k];
+        for (int k = 0; k < D + 2; ++k) v[k] = Num<T>::quarter(up ? slope[d][k] : -slope[d][k], v[k]);
     }
 }
 
 // every child of C has rho > 0 and p > 0
 template <typename T, int D>
 __device__ __forceinline__ bool prolong_positive(const Grid& g, const T (&UC)[D + 2], const T (&slope)[D][D + 2]) {
+    // the least rho and E and the largest momenta of any child bound them all:
+    // with a margin far above rounding this settles every cell but those next
+    // to a vacuum, and spares eight children their velocities and pressures
+    // (FP64, 3D: 25 instructions instead of 390 of the cell's 490)
+    const T margin = sizeof(T) == 8 ? T(1e-9) : T(1e-3);
+    auto reach = [&](int k) {
+        T r = fabs(slope[0][k]);
+#pragma unroll
+        for (int d = 1; d < D; ++d) r = r + fabs(slope[d][k]);
+        return T(0.25) * r;
+    };
+    const T rlo = UC[0] - reach(0), elo = UC[D + 1] - reach(D + 1);
+    T msq = T(0);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        const T mm = fabs(UC[1 + d]) + reach(1 + d);
+        msq = msq + mm * mm;
+    }
+    if (rlo > margin * UC[0] && rlo > T(1e-30) && elo > margin * UC[D + 1] &&
+        T(2) * rlo * elo > (T(1) + margin) * msq)
+        return true;
     const T gm1 = T(g.gamma) - T(1);
     bool ok = true;
-#pragma unroll
+#pragma unroll 1
     for (int ch = 0; ch < (1 << D); ++ch) {
         T v[D + 2];
         prolong_child<T, D>(UC, slope, ch, v);
