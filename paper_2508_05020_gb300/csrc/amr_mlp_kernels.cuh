@@ -57,33 +57,6 @@ cudaError_t Kernels<T>::harvest(const Grid& g, const T* U, int* n_out, double* s
     return cudaGetLastError();
 }
 
-template <typename T, int D, int N>
-__device__ bool plain_flag_cell(const Grid& g, const T* U, int slot, const int* l) {
-    constexpr int NV = D + 2;
-    const T gm1 = T(g.gamma) - T(1);
-    auto rho_p = [&](int dx, int dy, int dz, T& r, T& p) {
-        T Uc[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-            Uc[v] = U[slot_index(g, slot, v, sc<D>(2, l[2] + dz), sc<D>(1, l[1] + dy), sc<D>(0, l[0] + dx))];
-        T u[D], Tt;
-        primitives<T, D>(Uc, gm1, r, u, p, Tt);
-    };
-    T r0, p0;
-    rho_p(0, 0, 0, r0, p0);
-    bool f = false;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        const int ex = d == 0, ey = d == 1, ez = d == 2;
-        T rm, pm, rp, pp;
-        rho_p(-ex, -ey, -ez, rm, pm);
-        rho_p(ex, ey, ez, rp, pp);
-        f = f || (fabs(rp - rm) > T(g.theta_rho) * (rp + T(2) * r0 + rm)) ||
-            (fabs(pp - pm) > T(g.theta_p) * (pp + T(2) * p0 + pm));
-    }
-    return f;
-}
-
 // ---------------------------------------------------------------------------
 // K10: learned indicator on the band [-1, N]^d of every leaf patch. A work
 // item is a leaf patch (1D/2D) or a slab of DZ band planes of it (3D); items
