@@ -252,7 +252,8 @@ __global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
                     if (ks + PF < KS) fetch(ks + PF, wv[b]);
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
-                        const float x = Xs[r * K + kk];
+                        float x = Xs[r * K + kk];
+                        if (K % 32 != 0 && b == (KS - 1) % PF) x = k < K ? x : 0.f;   // not 0 * inf
 #pragma unroll
                         for (int j = 0; j < OW; ++j) acc[j * R + r] = fmaf(x, wk[j], acc[j * R + r]);
                     }
