@@ -346,7 +346,8 @@ int amr_harvest(amr_ctx* ctx, long* n, double* samples, uint8_t* labels);
  * [8] the ghost fill that precedes flagging (CUDA events), [9] the whole
  * flagging phase: ghost fill, flag kernel, request compaction and read-back
  * (wall). launches (may be NULL) receives the kernel launches behind each
- * slot (0 for the wall-clock slots). */
+ * slot (0 for the wall-clock slots). While it is enabled every class has
+ * launches of its own, so a small hierarchy's step takes a few launches more. */
 #define AMR_TIMING_SLOTS 10
 int amr_set_timing(amr_ctx* ctx, int enable);
 

@@ -533,11 +533,12 @@ int fill_all_levels(amr_ctx* c, T* U, double tfrac) {
 // Enqueue one SSP-RK3 step of the batched mode (optionally with the CFL step).
 // A small hierarchy's step is its launches (about 3 us each), so there are few:
 // one ghost fill for all levels (it reads interior cells only), dt set by the
-// CFL reduction's last block, the time moved on by the last RHS, no reflux with
-// one level: 13 launches with three levels where one per level and scalar made
-// 21 (1D FP32, four levels: 92 -> 51 us per step). Programmatic dependences between
-// them gained 1 to 3 %, and cost FP64 runs up to 40 %, as the early CTAs of an
-// RHS pile up on few SMs.
+// CFL reduction's last block; the finest level's
+// restriction in the RHS, the next level's with the flux correction; the time
+// moved on by the last RHS; no correction with one level. 10 launches with three
+// levels where one per level and scalar made 21 (1D FP32, four levels: 92 -> 43
+// us per step). Programmatic dependences between them gained 1 to 3 %, and cost
+// FP64 runs up to 40 %, as the early CTAs of an RHS pile up on few SMs.
 template <typename T>
 int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
     const Grid& g = c->grid;
@@ -547,19 +548,20 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
         return c->capturing ? cudaEventRecordWithFlags(e, c->stream, cudaEventRecordExternal)
                             : cudaEventRecord(e, c->stream);
     };
+    const int gghost = grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, true));
+    const int gcfl = grid_for(c, c->tune[AMR_TUNE_CFL_GRID], cfl_threads(c));
+    const bool merge = !c->timing;                        // with timing every class has launches of its own
     if (with_cfl) {
         CK(mark(c->ev_cfl[0]), "event");
-        CK(Kernels<T>::cfl(g, St<T>(c, 0), grid_for(c, c->tune[AMR_TUNE_CFL_GRID], cfl_threads(c)), c->stream, -1, true),
-           "cfl");
+        CK(Kernels<T>::cfl(g, St<T>(c, 0), gcfl, c->stream, -1, true), "cfl");
         CK(mark(c->ev_cfl[1]), "event");
         ++k;
     }
     const double tfrac[3] = {0.0, 1.0, 0.5};
     const RhsPlan plan = rhs_plan<T>(c);
-    const int gghost = grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, true));
     const int greflux = grid_for(c, c->tune[AMR_TUNE_REFLUX_GRID], 256);
     const int grestrict = grid_for(c, c->tune[AMR_TUNE_RESTRICT_GRID], restrict_threads(c));
-    const bool after = !c->timing && after_in_one(c);
+    const bool after = merge && after_in_one(c), settle = merge && c->L > 2;
     for (int s = 0; s < 3; ++s) {
         T* src = St<T>(c, s == 0 ? 0 : s);
         T* dst = St<T>(c, s == 0 ? 1 : (s == 1 ? 2 : 0));
@@ -584,12 +586,18 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
             }
             continue;
         }
-        if (c->L > 1) {
+        if (settle) {
+            CK(Kernels<T>::settle(g, dst, reinterpret_cast<T*>(c->faces), s,
+                                  grid_for(c, c->tune[AMR_TUNE_RESTRICT_GRID], 256), c->stream),
+               "settle");
+            ++k;
+        } else if (c->L > 1) {
             CK(Kernels<T>::reflux(g, dst, reinterpret_cast<T*>(c->faces), s, greflux, c->stream, -1), "reflux");
             ++k;
         }
         CK(mark(c->ev[s][3]), "event");
-        for (int l = c->L - 2; l >= 1; --l) {             // level L - 1: fused into the RHS
+        // level L - 1: fused into the RHS
+        for (int l = settle ? c->L - 3 : c->L - 2; l >= 1; --l) {
             CK(Kernels<T>::restrict_level(g, dst, l, grestrict, c->stream, -1), "restrict");
             ++k;
         }

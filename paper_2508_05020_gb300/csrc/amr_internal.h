@@ -157,6 +157,8 @@ struct Kernels {
     // covered cells of level-1 patches from the children of level `level`
     static cudaError_t restrict_level(const Grid& g, T* U, int level, int grid, cudaStream_t s,
                                       int one_slot);
+    // reflux and the restriction of level L - 2 (>= 1)
+    static cudaError_t settle(const Grid& g, T* U, const T* faces, int stage, int grid, cudaStream_t s);
     // reflux, the restriction of levels L - 2 .. 1 and (next) the next stage's
     // ghost fill of U in one launch, for a small 1D hierarchy
     static cudaError_t after_stage(const Grid& g, T* U, const T* faces, int stage, bool next, double tfrac, int chunk,

@@ -2015,6 +2015,46 @@ __global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int o
 }
 
 // ---------------------------------------------------------------------------
+// Three levels and more: the corrections of every level and the restriction of
+// level L - 2 in one launch. A patch of that level is restricted by the block
+// that corrected it (restricting it needs no other patch's correction: its
+// covered cells came from the finest level in the RHS), and the corrected cells
+// of coarser levels are leaves, which no restriction writes. Both are bound by
+// their dependent loads, so a launch of its own for each cost its latency: us per
+// step in FP32, separate launches / this one, 292 patches of 16^2 75.2 / 68.6,
+// 1024 of 32^2 91.0 / 84.8, 946 of 8^3 264 / 249, FP64 156 of 32^2 642 / 637.
+// ---------------------------------------------------------------------------
+template <typename T, int D, int N>
+__global__ void __launch_bounds__(256) k_settle(Grid g, T* U, const T* __restrict__ faces, int stage) {
+    const LaunchWords w(g);
+    const int level = g.L - 2;
+    const int lo = g.level_off[level], n_lev = g.level_off[level + 1] - lo;
+    if (w.cancel) return;
+    const T dt = T(w.dt);
+    for (int item = blockIdx.x; item < w.n_reflux + n_lev; item += gridDim.x) {
+        int slot;
+        if (item < w.n_reflux) {
+            reflux_patch<T, D, N>(g, U, faces, stage_b<T>(stage), dt, item);
+            slot = g.reflux_list[item];
+            if (g.level[slot] != level) continue;
+            __syncthreads();                             // its corrected cells are read below
+        } else {
+            slot = g.all_list[lo + item - w.n_reflux];
+            // a leaf with a face next to a patch with children is in the list
+            const int f = threadIdx.x;
+            int listed = 0;
+            if (f < 2 * D && !(g.pflag[slot] & 1)) {
+                const int d = f >> 1;
+                const int nb = g.nbr[slot * NBR + 13 + ((f & 1) ? 1 : -1) * (d == 0 ? 1 : (d == 1 ? 3 : 9))];
+                listed = nb >= 0 && (g.pflag[nb] & 1);
+            }
+            if (__syncthreads_or(listed)) continue;
+        }
+        restrict_items<T, D, N>(g, U, 0, 0, slot, threadIdx.x, 256);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // What follows the RHS of a stage, for a small 1D hierarchy, in one launch of one
 // cluster: the flux correction, the restriction level by level and the next
 // stage's ghost fill, with the cluster's barrier where a launch

@@ -302,6 +302,12 @@ cudaError_t Kernels<T>::restrict_level(const Grid& g, T* U, int level, int grid,
 }
 
 template <typename T>
+cudaError_t Kernels<T>::settle(const Grid& g, T* U, const T* faces, int stage, int grid, cudaStream_t s) {
+    AMR_DISPATCH(g, (k_settle<T, D, N><<<grid, 256, 0, s>>>(g, U, faces, stage)));
+    return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t Kernels<T>::after_stage(const Grid& g, T* U, const T* faces, int stage, bool next, double tfrac, int chunk,
                                     cudaStream_t s) {
     auto go = [&](auto n) {
