@@ -532,10 +532,10 @@ int fill_all_levels(amr_ctx* c, T* U, double tfrac) {
 
 // Enqueue one SSP-RK3 step of the batched mode (optionally with the CFL step).
 // A small hierarchy's step is its launches (about 3 us each), so there are few:
-// one ghost fill for all levels (it reads interior cells only), dt set by the
-// CFL reduction's last block; the finest level's
+// one ghost fill for all levels (it reads interior cells only), the first one
+// together with the CFL reduction, whose last block sets dt; the finest level's
 // restriction in the RHS, the next level's with the flux correction; the time
-// moved on by the last RHS; no correction with one level. 10 launches with three
+// moved on by the last RHS; no correction with one level. 9 launches with three
 // levels where one per level and scalar made 21 (1D FP32, four levels: 92 -> 43
 // us per step). Programmatic dependences between them gained 1 to 3 %, and cost
 // FP64 runs up to 40 %, as the early CTAs of an RHS pile up on few SMs.
@@ -551,7 +551,12 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
     const int gghost = grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, true));
     const int gcfl = grid_for(c, c->tune[AMR_TUNE_CFL_GRID], cfl_threads(c));
     const bool merge = !c->timing;                        // with timing every class has launches of its own
-    if (with_cfl) {
+    const bool begin = merge && with_cfl && !skip_fill0;
+    if (begin) {
+        CK(Kernels<T>::begin_step(g, St<T>(c, 0), gcfl, gcfl + gghost, c->tune[AMR_TUNE_GHOST_CHUNK], c->stream),
+           "begin step");
+        ++k;
+    } else if (with_cfl) {
         CK(mark(c->ev_cfl[0]), "event");
         CK(Kernels<T>::cfl(g, St<T>(c, 0), gcfl, c->stream, -1, true), "cfl");
         CK(mark(c->ev_cfl[1]), "event");
@@ -566,7 +571,7 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
         T* src = St<T>(c, s == 0 ? 0 : s);
         T* dst = St<T>(c, s == 0 ? 1 : (s == 1 ? 2 : 0));
         CK(mark(c->ev[s][0]), "event");
-        if (s == 0 ? !skip_fill0 : !after) {
+        if (s == 0 ? !skip_fill0 && !begin : !after) {
             CK(Kernels<T>::ghost_fill(g, src, tfrac[s], gghost, c->stream, -1, c->tune[AMR_TUNE_GHOST_CHUNK], true),
                "ghost fill");
             ++k;

@@ -157,6 +157,9 @@ struct Kernels {
     // covered cells of level-1 patches from the children of level `level`
     static cudaError_t restrict_level(const Grid& g, T* U, int level, int grid, cudaStream_t s,
                                       int one_slot);
+    // the CFL reduction with the step (ncfl blocks of the grid) and the stage fill
+    // of U at the time t
+    static cudaError_t begin_step(const Grid& g, T* U, int ncfl, int grid, int chunk, cudaStream_t s);
     // reflux and the restriction of level L - 2 (>= 1)
     static cudaError_t settle(const Grid& g, T* U, const T* faces, int stage, int grid, cudaStream_t s);
     // reflux, the restriction of levels L - 2 .. 1 and (next) the next stage's

@@ -302,6 +302,13 @@ cudaError_t Kernels<T>::restrict_level(const Grid& g, T* U, int level, int grid,
 }
 
 template <typename T>
+cudaError_t Kernels<T>::begin_step(const Grid& g, T* U, int ncfl, int grid, int chunk, cudaStream_t s) {
+    AMR_DISPATCH(g, (k_begin<T, D, N><<<grid, 256, 0, s>>>(g, U, ncfl, d4(g.dmr_pre), d4(g.dmr_post), chunk,
+                                                           g.n_ghost_face)));
+    return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t Kernels<T>::settle(const Grid& g, T* U, const T* faces, int stage, int grid, cudaStream_t s) {
     AMR_DISPATCH(g, (k_settle<T, D, N><<<grid, 256, 0, s>>>(g, U, faces, stage)));
     return cudaGetLastError();

@@ -1,6 +1,7 @@
 """The launches of a step that hold two kernels' work, against the same step
 with a launch for each (device timing on): the flux correction with the
-restriction of the level below the finest. Both forms run the same device functions in an order
+restriction of the level below the finest, and the CFL reduction with the
+first stage's ghost fill. Both forms run the same device functions in an order
 that no result depends on, so every cell is the same to the last bit.
 
 Hierarchies with three and four levels, where leaves border on finer patches
