@@ -148,7 +148,8 @@ typedef struct {
  * SM of the fused RHS, the reflux, the restriction, the CFL reduction and the
  * plain flagging. Until amr_autotune or amr_set_tuning chooses another RHS
  * grid or tile shape than the default (2, 0), the RHS's grid follows a rule of
- * the library by precision, dimension and patch size. */
+ * the library by precision, dimension and patch size. The same holds for the
+ * ghost fill's grid and work items (16, 128). */
 #define AMR_TUNE_GHOST_GRID 0
 #define AMR_TUNE_GHOST_CHUNK 1
 #define AMR_TUNE_RHS_GRID 2

@@ -71,8 +71,9 @@ struct amr_ctx {
     int tune[AMR_TUNE_N] = {16, 128, 2, 4, 8, 8, 4, 0};
     float tune_ms[AMR_TUNE_N] = {0, 0, 0, 0, 0, 0, 0, 0};
     // the RHS's grid and tile shape were chosen (autotuner, amr_set_tuning);
-    // before that its grid follows the kernel's own rule (Kernels::rhs_grid)
-    bool rhs_tuned = false;
+    // before that its grid follows the kernel's own rule (Kernels::rhs_grid);
+    // the same for the grid and work items of the ghost fill (ghost_ctas, ghost_chunk)
+    bool rhs_tuned = false, ghost_tuned = false;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     // hierarchy
@@ -443,10 +444,27 @@ int grid_for(const amr_ctx* c, int per_sm, long long per_patch) {
     const long long most = std::min<long long>(1ll << size_bits(c), c->cap);
     return (int)std::max<long long>(1, std::min<long long>(grid_size(c, per_sm), (most * per_patch + 255) / 256));
 }
+// A stage's ghost fill in 2D from 4096 patches on looks at 32 boxes at a time
+// (`look`), with 4 CTAs per SM unless they were chosen: us per step in FP32, 25600
+// patches of 16^2 1230 -> 1151, 4096 of 8^2 154 -> 129, 16384 360 -> 344 (these with
+// 16 CTAs). Below, every warp has one box and looking ahead costs 1 to 3 %; in 3D
+// it changes nothing (1536 patches of 16^3 1920 / 1913).
+bool ghost_look(const amr_ctx* c) { return c->dim == 2 && size_bits(c) > 12; }
+int ghost_ctas(const amr_ctx* c) {
+    return ghost_look(c) && !c->ghost_tuned ? 4 : c->tune[AMR_TUNE_GHOST_GRID];
+}
+// Ghost cells per work item of a stage's fill: a whole face box of an 8^3 patch,
+// whose 32 coarse cells are one pass of a warp, where the boxes outnumber the
+// resident warps, unless it was chosen (FP32, us per step, 128 cells / a box:
+// 946 patches 246 / 235; but 83 patches 89.1 / 92.4)
+int ghost_chunk(const amr_ctx* c) {
+    const bool box = c->dim == 3 && c->N == 8 && size_bits(c) > 9 && !c->ghost_tuned;
+    return box ? 3 * 8 * 8 : c->tune[AMR_TUNE_GHOST_CHUNK];
+}
 // threads per patch of the ghost fills (a warp per work item), the CFL
 // reduction (16-byte vectors of cells) and the restriction (coarse cells)
 long long ghost_threads(const amr_ctx* c, bool stage_only) {
-    const int chunk = c->tune[AMR_TUNE_GHOST_CHUNK];
+    const int chunk = stage_only ? ghost_chunk(c) : c->tune[AMR_TUNE_GHOST_CHUNK];
     const int face = c->n_ghost_face / (2 * c->dim);
     return 32ll * (stage_only ? 2 * c->dim * ((face + chunk - 1) / chunk) : (c->n_ghost + chunk - 1) / chunk);
 }
@@ -548,12 +566,13 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
         return c->capturing ? cudaEventRecordWithFlags(e, c->stream, cudaEventRecordExternal)
                             : cudaEventRecord(e, c->stream);
     };
-    const int gghost = grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, true));
+    const int gghost = grid_for(c, ghost_ctas(c), ghost_threads(c, true));
+    const bool look = ghost_look(c);
     const int gcfl = grid_for(c, c->tune[AMR_TUNE_CFL_GRID], cfl_threads(c));
     const bool merge = !c->timing;                        // with timing every class has launches of its own
     const bool begin = merge && with_cfl && !skip_fill0;
     if (begin) {
-        CK(Kernels<T>::begin_step(g, St<T>(c, 0), gcfl, gcfl + gghost, c->tune[AMR_TUNE_GHOST_CHUNK], c->stream),
+        CK(Kernels<T>::begin_step(g, St<T>(c, 0), gcfl, gcfl + gghost, ghost_chunk(c), look, c->stream),
            "begin step");
         ++k;
     } else if (with_cfl) {
@@ -572,7 +591,7 @@ int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
         T* dst = St<T>(c, s == 0 ? 1 : (s == 1 ? 2 : 0));
         CK(mark(c->ev[s][0]), "event");
         if (s == 0 ? !skip_fill0 && !begin : !after) {
-            CK(Kernels<T>::ghost_fill(g, src, tfrac[s], gghost, c->stream, -1, c->tune[AMR_TUNE_GHOST_CHUNK], true),
+            CK(Kernels<T>::ghost_fill(g, src, tfrac[s], gghost, c->stream, -1, ghost_chunk(c), true, look),
                "ghost fill");
             ++k;
         }
@@ -1114,13 +1133,14 @@ int autotune_impl(amr_ctx* c) {
                 float t = 0.f;
                 err = timed([&]() {
                     ++nk;
-                    return Kernels<T>::ghost_fill(g, A, 0.0, grid_size(c, gr), c->stream, -1, ch, true);
+                    return Kernels<T>::ghost_fill(g, A, 0.0, grid_size(c, gr), c->stream, -1, ch, true, ghost_look(c));
                 }, t);
                 if (err != cudaSuccess) break;
                 if (t < bestv) {
                     bestv = t;
                     c->tune[AMR_TUNE_GHOST_GRID] = gr;
                     c->tune[AMR_TUNE_GHOST_CHUNK] = ch;
+                    c->ghost_tuned = true;
                 }
             }
         c->tune_ms[AMR_TUNE_GHOST_GRID] = c->tune_ms[AMR_TUNE_GHOST_CHUNK] = bestv;
@@ -1788,7 +1808,9 @@ int amr_set_tuning(amr_ctx* c, const int params[AMR_TUNE_N]) {
         else ok = v >= 1 && v <= 64;
         if (!ok) return fail(c, AMR_ERR_ARG, "launch parameter out of range");
     }
-    // the values an untuned context reports, set again, leave the RHS untuned
+    // the values an untuned context reports, set again, leave it untuned
+    c->ghost_tuned = c->ghost_tuned || params[AMR_TUNE_GHOST_GRID] != c->tune[AMR_TUNE_GHOST_GRID] ||
+                     params[AMR_TUNE_GHOST_CHUNK] != c->tune[AMR_TUNE_GHOST_CHUNK];
     c->rhs_tuned = c->rhs_tuned || params[AMR_TUNE_RHS_GRID] != c->tune[AMR_TUNE_RHS_GRID] ||
                    params[AMR_TUNE_RHS_SHAPE] != c->tune[AMR_TUNE_RHS_SHAPE];
     for (int i = 0; i < AMR_TUNE_N; ++i) c->tune[i] = params[i];

@@ -139,8 +139,10 @@ struct Kernels {
     // face (all a stage reads from a slot's ghost region: the RHS and the
     // prolongation read same-level neighbours' interiors directly); else every
     // ghost cell (what the flag stencils read)
+    // look: the stage's form for a large hierarchy (2D)
     static cudaError_t ghost_fill(const Grid& g, T* U, double tfrac, int grid,
-                                  cudaStream_t s, int one_slot, int chunk = 512, bool stage_only = false);
+                                  cudaStream_t s, int one_slot, int chunk = 512, bool stage_only = false,
+                                  bool look = false);
     // compiled tile-shape candidates of the fused RHS for this grid and flux
     static int rhs_shapes(const Grid& g);
     // how a hierarchy of `leaves` leaf patches (in a pool of g.cap) is advanced with tile shape 0
@@ -159,7 +161,7 @@ struct Kernels {
                                       int one_slot);
     // the CFL reduction with the step (ncfl blocks of the grid) and the stage fill
     // of U at the time t
-    static cudaError_t begin_step(const Grid& g, T* U, int ncfl, int grid, int chunk, cudaStream_t s);
+    static cudaError_t begin_step(const Grid& g, T* U, int ncfl, int grid, int chunk, bool look, cudaStream_t s);
     // reflux and the restriction of level L - 2 (>= 1)
     static cudaError_t settle(const Grid& g, T* U, const T* faces, int stage, int grid, cudaStream_t s);
     // reflux, the restriction of levels L - 2 .. 1 and (next) the next stage's

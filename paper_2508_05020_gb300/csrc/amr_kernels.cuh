@@ -1026,8 +1026,12 @@ __device__ void ghost_value(const Grid& g, const T* U, const PatchMeta& m, int* 
 // `chunk` cells (the size is a launch parameter chosen by the autotuner),
 // taken by one warp, which stages the patch's metadata in its own
 // shared-memory copy; warps never wait for one another.
+// A stage of a large hierarchy skips most boxes, and a warp that looks at them
+// one after the other waits for two dependent loads per box (41 us for 25600
+// patches of 16^2). With LOOK each lane looks at one of the warp's next 32
+// items, and the warp works through those with something to fill.
 // ---------------------------------------------------------------------------
-template <typename T, int D, int N, bool STAGE>
+template <typename T, int D, int N, bool STAGE, bool LOOK = false>
 __device__ __forceinline__ void ghost_items(const Grid& g, T* U, double t, int n_all, int one_slot, double4 pre,
                                             double4 post, int chunk, int n_cells, int warp, int nw, PatchMeta& m) {
     constexpr bool stage_only = STAGE;                  // compiled apart: the full fill keeps its registers
@@ -1044,7 +1048,21 @@ __device__ __forceinline__ void ghost_items(const Grid& g, T* U, double t, int n
     const int span = stage_only ? BOX : n_cells;          // table entries one run of items covers
     const int nruns = stage_only ? 2 * D : 1;
     const int nchunk = (span + chunk - 1) / chunk;        // chunk: ghost cells per work item
-    for (int item = warp; item < npatch * nruns * nchunk; item += nw) {
+    const int total = npatch * nruns * nchunk;
+    for (int first = warp; first < total; first += LOOK ? 32 * nw : nw) {
+        unsigned todo = 1;                                // of the items first + k nw, those to be done
+        if constexpr (LOOK) {
+            bool fill = false;
+            if (total - first > lane * nw) {
+                const int item = first + lane * nw;
+                const int d = item % (nruns * nchunk) / nchunk;
+                const int slot = one_slot >= 0 ? one_slot : g.all_list[item / (nruns * nchunk)];
+                fill = g.nbr[slot * NBR + 13 + ((d & 1) ? 1 : -1) * (d < 2 ? 1 : (d < 4 ? 3 : 9))] < 0;
+            }
+            todo = __ballot_sync(0xFFFFFFFFu, fill);
+        }
+        for (; todo; todo &= todo - 1) {
+        const int item = first + (LOOK ? __ffs(todo) - 1 : 0) * nw;
         const int pi = item / (nruns * nchunk);
         const int rest = item - pi * nruns * nchunk;
         const int run = rest / nchunk;
@@ -1129,17 +1147,18 @@ __device__ __forceinline__ void ghost_items(const Grid& g, T* U, double t, int n
             for (int v = 0; v < NV; ++v) U[slot_index(g, slot, v, sz, sy, sx)] = val[v];
         }
         __syncwarp();                                    // the copy is read until here
+        }
     }
 }
 
-template <typename T, int D, int N, bool STAGE>
+template <typename T, int D, int N, bool STAGE, bool LOOK = false>
 __global__ void __launch_bounds__(256, STAGE && sizeof(T) == 4 ? 3 : 0) k_ghost(Grid g, T* U, double tfrac, int one_slot,
                                                double4 pre, double4 post, int chunk, int n_cells) {
     __shared__ PatchMeta metas[256 / 32];
     const LaunchWords w(g);
     if (w.cancel) return;
     const int warp = threadIdx.x >> 5;
-    ghost_items<T, D, N, STAGE>(g, U, w.t + tfrac * w.dt, w.n_all, one_slot, pre, post, chunk, n_cells,
+    ghost_items<T, D, N, STAGE, LOOK>(g, U, w.t + tfrac * w.dt, w.n_all, one_slot, pre, post, chunk, n_cells,
                                 blockIdx.x * (256 / 32) + warp, gridDim.x * (256 / 32), metas[warp]);
 }
 
@@ -2022,7 +2041,7 @@ __global__ void __launch_bounds__(256) k_restrict(Grid g, T* U, int level, int o
 // of coarser levels are leaves, which no restriction writes. Both are bound by
 // their dependent loads, so a launch of its own for each cost its latency: us per
 // step in FP32, separate launches / this one, 292 patches of 16^2 75.2 / 68.6,
-// 1024 of 32^2 91.0 / 84.8, 946 of 8^3 264 / 249, FP64 156 of 32^2 642 / 637.
+// 1024 91.0 / 84.8, 946 of 8^3 264 / 249, FP64 156 of 16^2 642 / 637.
 // ---------------------------------------------------------------------------
 template <typename T, int D, int N>
 __global__ void __launch_bounds__(256) k_settle(Grid g, T* U, const T* __restrict__ faces, int stage) {
@@ -2186,8 +2205,8 @@ __global__ void __launch_bounds__(256) k_cfl(Grid g, const T* U, int one_slot, i
 // launch, and neither waits for the other. It writes ghost cells, which the
 // reduction does not read. Us per step, two launches / one: FP32 496 patches of
 // 8^2 60.3 / 54.5, 72 of 8^3 72.7 / 68.9, 25600 of 16^2 1242 / 1233; FP64 12
-// patches of 1D 74.1 / 68.0, 76 of 8^2 189 / 178, 992 of 32^2 2540 / 2540.
-template <typename T, int D, int N>
+// patches of 1D 74.1 / 68.0, 76 of 8^2 189 / 178, 992 of 16^2 2540 / 2540.
+template <typename T, int D, int N, bool LOOK = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 0)
     k_begin(Grid g, T* U, int ncfl, double4 pre, double4 post, int chunk, int n_cells) {
     __shared__ PatchMeta metas[256 / 32];
@@ -2197,7 +2216,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 0)
         cfl_cells<T, D, N>(g, U, w.n_leaf, -1, 1, blockIdx.x, ncfl);
     } else {
         const int warp = threadIdx.x >> 5;
-        ghost_items<T, D, N, true>(g, U, w.t, w.n_all, -1, pre, post, chunk, n_cells,
+        ghost_items<T, D, N, true, LOOK>(g, U, w.t, w.n_all, -1, pre, post, chunk, n_cells,
                                    ((int)blockIdx.x - ncfl) * (256 / 32) + warp, ((int)gridDim.x - ncfl) * (256 / 32),
                                    metas[warp]);
     }

@@ -267,10 +267,13 @@ cudaError_t Kernels<T>::prepare(const Grid& g) {
 
 template <typename T>
 cudaError_t Kernels<T>::ghost_fill(const Grid& g, T* U, double tfrac, int grid, cudaStream_t s, int one_slot,
-                                   int chunk, bool stage_only) {
+                                   int chunk, bool stage_only, bool look) {
     if (chunk < 32) return cudaErrorInvalidValue;
     const int n_cells = stage_only ? g.n_ghost_face : g.n_ghost;
-    if (stage_only) {
+    if (stage_only && look) {
+        AMR_DISPATCH(g, (k_ghost<T, D, N, true, D == 2><<<grid, 256, 0, s>>>(g, U, tfrac, one_slot, d4(g.dmr_pre),
+                                                                              d4(g.dmr_post), chunk, n_cells)));
+    } else if (stage_only) {
         AMR_DISPATCH(g, (k_ghost<T, D, N, true><<<grid, 256, 0, s>>>(g, U, tfrac, one_slot, d4(g.dmr_pre),
                                                                       d4(g.dmr_post), chunk, n_cells)));
     } else {
@@ -302,9 +305,14 @@ cudaError_t Kernels<T>::restrict_level(const Grid& g, T* U, int level, int grid,
 }
 
 template <typename T>
-cudaError_t Kernels<T>::begin_step(const Grid& g, T* U, int ncfl, int grid, int chunk, cudaStream_t s) {
-    AMR_DISPATCH(g, (k_begin<T, D, N><<<grid, 256, 0, s>>>(g, U, ncfl, d4(g.dmr_pre), d4(g.dmr_post), chunk,
-                                                           g.n_ghost_face)));
+cudaError_t Kernels<T>::begin_step(const Grid& g, T* U, int ncfl, int grid, int chunk, bool look, cudaStream_t s) {
+    if (look) {
+        AMR_DISPATCH(g, (k_begin<T, D, N, D == 2><<<grid, 256, 0, s>>>(g, U, ncfl, d4(g.dmr_pre), d4(g.dmr_post),
+                                                                        chunk, g.n_ghost_face)));
+    } else {
+        AMR_DISPATCH(g, (k_begin<T, D, N><<<grid, 256, 0, s>>>(g, U, ncfl, d4(g.dmr_pre), d4(g.dmr_post), chunk,
+                                                               g.n_ghost_face)));
+    }
     return cudaGetLastError();
 }
 
