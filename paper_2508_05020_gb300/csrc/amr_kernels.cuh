@@ -2282,7 +2282,11 @@ __device__ bool plain_flag_cell(const Grid& g, const T* U, int slot, const int* 
     return f;
 }
 
-// FP64: rho, p and a bound on p's error of one cell in FP32
+// FP64: rho, p and a bound on p's error of one cell in FP32. The bound holds at
+// any scale: relative, for the roundings of normal numbers, and absolute, for
+// squares, sums and quotients that fall below the FP32 range (each off by less
+// than 1e-45, the squared momentum's error divided by rho). A density so small
+// that its reciprocal overflows makes it infinite or NaN, which settles nothing.
 struct SensorCell {
     float rho, p, err;
 };
@@ -2295,8 +2299,9 @@ __device__ __forceinline__ SensorCell sensor_cell(const double (&U)[D + 2], floa
         const float m = (float)U[1 + d];
         msq = fmaf(m, m, msq);
     }
-    const float ke = 0.5f * msq / rho;
-    return {rho, gm1 * (E - ke), 2.0e-6f * gm1 * (fabsf(E) + fabsf(ke))};
+    const float r = 1.0f / rho;
+    const float ke = 0.5f * msq * r;
+    return {rho, gm1 * (E - ke), gm1 * fmaf(2.0e-6f, fabsf(E) + fabsf(ke), 1.0e-44f * (1.0f + fabsf(r)))};
 }
 // |a - b| > th (a + 2 c + b) for values known to within e in all (their errors
 // summed with these weights): 1 surely, -1 surely not, 0 not settled
