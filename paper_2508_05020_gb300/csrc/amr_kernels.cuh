@@ -848,7 +848,10 @@ __device__ __forceinline__ void prolong_slopes(const Grid& g, const T* U, int Q,
         bool mirror = false, isfixed = false;
         if (NBR_READS && (outp || outm)) {
             const int kind = g.bc[d][outp ? 1 : 0];
-            if constexpr (D == 2) isfixed = bc_fixed<T, D>(g, kind, g.level[Q], g.coord[Q * 3] * N + Lc[0], bc, fixed);
+            if constexpr (D == 2) {                      // the ghost's own x: next to C's across an x side
+                const int gx = g.coord[Q * 3] * N + Lc[0] + (d == 0 ? (outp ? 1 : -1) : 0);
+                isfixed = bc_fixed<T, D>(g, kind, g.level[Q], gx, bc, fixed);
+            }
             mirror = !isfixed && kind != AMR_BC_OUTFLOW;
         }
 #pragma unroll
