@@ -909,8 +909,10 @@ __device__ __forceinline__ bool prolong_positive(const Grid& g, const T (&UC)[D 
         const T mm = fabs(UC[1 + d]) + reach(1 + d);
         msq = msq + mm * mm;
     }
-    if (rlo > margin * UC[0] && rlo > T(1e-30) && elo > margin * UC[D + 1] &&
-        T(2) * rlo * elo > (T(1) + margin) * msq)
+    // (products near the subnormals have no digits left for the margin)
+    const T least = sizeof(T) == 8 ? T(1e-290) : T(1e-35);
+    const T re = T(2) * rlo * elo;
+    if (rlo > margin * UC[0] && rlo > T(1e-30) && elo > margin * UC[D + 1] && re > least && re > (T(1) + margin) * msq)
         return true;
     const T gm1 = T(g.gamma) - T(1);
     bool ok = true;
