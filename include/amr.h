@@ -149,7 +149,8 @@ typedef struct {
  * plain flagging. Until amr_autotune or amr_set_tuning chooses another RHS
  * grid or tile shape than the default (2, 0), the RHS's grid follows a rule of
  * the library by precision, dimension and patch size. The same holds for the
- * ghost fill's grid and work items (16, 128). */
+ * ghost fill's grid and work items (16, 128). These two are a stage's fill; the
+ * full fill of a regrid takes 16 and 128 until amr_set_tuning sets another pair. */
 #define AMR_TUNE_GHOST_GRID 0
 #define AMR_TUNE_GHOST_CHUNK 1
 #define AMR_TUNE_RHS_GRID 2

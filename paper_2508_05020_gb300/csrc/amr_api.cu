@@ -71,9 +71,14 @@ struct amr_ctx {
     int tune[AMR_TUNE_N] = {16, 128, 2, 4, 8, 8, 4, 0};
     float tune_ms[AMR_TUNE_N] = {0, 0, 0, 0, 0, 0, 0, 0};
     // the RHS's grid and tile shape were chosen (autotuner, amr_set_tuning);
-    // before that its grid follows the kernel's own rule (Kernels::rhs_grid);
-    // the same for the grid and work items of the ghost fill (ghost_ctas, ghost_chunk)
+    // before that its grid follows the kernel's own rule (Kernels::rhs_plan);
+    // the same for the grid and work items of a stage's ghost fill (ghost_ctas, ghost_chunk)
     bool rhs_tuned = false, ghost_tuned = false;
+    // CTAs per SM and ghost cells per work item of a regrid's full ghost fill. The
+    // autotuner measures a stage's fill, whose best items (whole face boxes) are
+    // too large for this one: 128^3 blast, 1536 patches, 286 us with these, 306 to
+    // 324 with the stage's choice of 256 or 512 cells
+    int fill_ctas = 16, fill_chunk = 128;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     // hierarchy
@@ -464,7 +469,7 @@ int ghost_chunk(const amr_ctx* c) {
 // threads per patch of the ghost fills (a warp per work item), the CFL
 // reduction (16-byte vectors of cells) and the restriction (coarse cells)
 long long ghost_threads(const amr_ctx* c, bool stage_only) {
-    const int chunk = stage_only ? ghost_chunk(c) : c->tune[AMR_TUNE_GHOST_CHUNK];
+    const int chunk = stage_only ? ghost_chunk(c) : c->fill_chunk;
     const int face = c->n_ghost_face / (2 * c->dim);
     return 32ll * (stage_only ? 2 * c->dim * ((face + chunk - 1) / chunk) : (c->n_ghost + chunk - 1) / chunk);
 }
@@ -540,9 +545,8 @@ bool encode_tmaps(amr_ctx* c) {
 
 template <typename T>
 int fill_all_levels(amr_ctx* c, T* U, double tfrac) {
-    CK(Kernels<T>::ghost_fill(c->grid, U, tfrac,
-                              grid_for(c, c->tune[AMR_TUNE_GHOST_GRID], ghost_threads(c, false)), c->stream, -1,
-                              c->tune[AMR_TUNE_GHOST_CHUNK]),
+    CK(Kernels<T>::ghost_fill(c->grid, U, tfrac, grid_for(c, c->fill_ctas, ghost_threads(c, false)), c->stream, -1,
+                              c->fill_chunk),
        "ghost fill");
     ++c->kernels;
     return AMR_OK;
@@ -1813,6 +1817,11 @@ int amr_set_tuning(amr_ctx* c, const int params[AMR_TUNE_N]) {
                      params[AMR_TUNE_GHOST_CHUNK] != c->tune[AMR_TUNE_GHOST_CHUNK];
     c->rhs_tuned = c->rhs_tuned || params[AMR_TUNE_RHS_GRID] != c->tune[AMR_TUNE_RHS_GRID] ||
                    params[AMR_TUNE_RHS_SHAPE] != c->tune[AMR_TUNE_RHS_SHAPE];
+    if (params[AMR_TUNE_GHOST_GRID] != c->tune[AMR_TUNE_GHOST_GRID] ||
+        params[AMR_TUNE_GHOST_CHUNK] != c->tune[AMR_TUNE_GHOST_CHUNK]) {   // asked for: both fills
+        c->fill_ctas = params[AMR_TUNE_GHOST_GRID];
+        c->fill_chunk = params[AMR_TUNE_GHOST_CHUNK];
+    }
     for (int i = 0; i < AMR_TUNE_N; ++i) c->tune[i] = params[i];
     c->grid.rhs_shape = c->tune[AMR_TUNE_RHS_SHAPE];
     drop_graphs(c);
