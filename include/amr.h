@@ -146,11 +146,12 @@ typedef struct {
 /* Launch parameters of the batched step (amr_get_tuning), in this order:
  * CTAs per SM of the ghost fill, ghost cells per ghost-fill work item, CTAs per
  * SM of the fused RHS, the reflux, the restriction, the CFL reduction and the
- * plain flagging. Until amr_autotune or amr_set_tuning chooses another RHS
- * grid or tile shape than the default (2, 0), the RHS's grid follows a rule of
- * the library by precision, dimension and patch size. The same holds for the
- * ghost fill's grid and work items (16, 128). These two are a stage's fill; the
- * full fill of a regrid takes 16 and 128 until amr_set_tuning sets another pair. */
+ * plain flagging. Until amr_autotune or amr_set_tuning is called, the RHS's
+ * grid follows a rule of the library by precision, dimension, patch size and
+ * leaf count, the ghost fill's grid and work items one by dimension, patch size
+ * and patch count; amr_get_tuning reports what they give the present hierarchy.
+ * The ghost fill's two are a stage's; the full fill of a regrid takes 16 and 128
+ * until amr_set_tuning sets a pair other than the one in use. */
 #define AMR_TUNE_GHOST_GRID 0
 #define AMR_TUNE_GHOST_CHUNK 1
 #define AMR_TUNE_RHS_GRID 2
@@ -369,7 +370,8 @@ int amr_autotune(amr_ctx* ctx);
 int amr_get_tuning(amr_ctx* ctx, int params[AMR_TUNE_N], float ms[AMR_TUNE_N]);
 /* Set the launch parameters (AMR_TUNE_N ints in AMR_TUNE_* order, as
  * amr_get_tuning returns them), for instance to reuse an earlier autotune's
- * choice. CTAs per SM in [1, 64], ghost cells per work item in [32, 4096],
+ * choice. All of them are launched as given from then on, whatever the hierarchy
+ * becomes. CTAs per SM in [1, 64], ghost cells per work item in [32, 4096],
  * the RHS tile shape below the number of compiled candidates; otherwise
  * AMR_ERR_ARG and nothing changes. Results do not depend on the choice. */
 int amr_set_tuning(amr_ctx* ctx, const int params[AMR_TUNE_N]);

@@ -337,7 +337,8 @@ class AMR:
 
     def set_tuning(self, params):
         """Set the launch parameters (a dict by TUNE_NAMES, as tuning() returns
-        them; missing names keep their value) (amr_set_tuning)."""
+        them; missing names keep the value in use) (amr_set_tuning). From then
+        on none of them follows the hierarchy."""
         cur, _ = self.tuning()
         cur.update(params)
         p = np.array([cur[k] for k in TUNE_NAMES], dtype=np.int32)

@@ -70,7 +70,8 @@ struct amr_ctx {
     // item), the defaults or the autotuner's choice (AMR_TUNE_* order)
     int tune[AMR_TUNE_N] = {16, 128, 2, 4, 8, 8, 4, 0};
     float tune_ms[AMR_TUNE_N] = {0, 0, 0, 0, 0, 0, 0, 0};
-    // the RHS's grid and tile shape were chosen (autotuner, amr_set_tuning);
+    // the RHS's grid and tile shape were chosen (autotuner, amr_set_tuning: any
+    // value that is set, the default ones too, is launched from then on);
     // before that its grid follows the kernel's own rule (Kernels::rhs_plan);
     // the same for the grid and work items of a stage's ghost fill (ghost_ctas, ghost_chunk)
     bool rhs_tuned = false, ghost_tuned = false;
@@ -1812,16 +1813,11 @@ int amr_set_tuning(amr_ctx* c, const int params[AMR_TUNE_N]) {
         else ok = v >= 1 && v <= 64;
         if (!ok) return fail(c, AMR_ERR_ARG, "launch parameter out of range");
     }
-    // the values an untuned context reports, set again, leave it untuned
-    c->ghost_tuned = c->ghost_tuned || params[AMR_TUNE_GHOST_GRID] != c->tune[AMR_TUNE_GHOST_GRID] ||
-                     params[AMR_TUNE_GHOST_CHUNK] != c->tune[AMR_TUNE_GHOST_CHUNK];
-    c->rhs_tuned = c->rhs_tuned || params[AMR_TUNE_RHS_GRID] != c->tune[AMR_TUNE_RHS_GRID] ||
-                   params[AMR_TUNE_RHS_SHAPE] != c->tune[AMR_TUNE_RHS_SHAPE];
-    if (params[AMR_TUNE_GHOST_GRID] != c->tune[AMR_TUNE_GHOST_GRID] ||
-        params[AMR_TUNE_GHOST_CHUNK] != c->tune[AMR_TUNE_GHOST_CHUNK]) {   // asked for: both fills
-        c->fill_ctas = params[AMR_TUNE_GHOST_GRID];
+    if (params[AMR_TUNE_GHOST_GRID] != ghost_ctas(c) || params[AMR_TUNE_GHOST_CHUNK] != ghost_chunk(c)) {
+        c->fill_ctas = params[AMR_TUNE_GHOST_GRID];          // another pair than in use: both fills
         c->fill_chunk = params[AMR_TUNE_GHOST_CHUNK];
     }
+    c->rhs_tuned = c->ghost_tuned = true;
     for (int i = 0; i < AMR_TUNE_N; ++i) c->tune[i] = params[i];
     c->grid.rhs_shape = c->tune[AMR_TUNE_RHS_SHAPE];
     drop_graphs(c);
@@ -1834,6 +1830,11 @@ int amr_get_tuning(amr_ctx* c, int params[AMR_TUNE_N], float ms[AMR_TUNE_N]) {
         params[i] = c->tune[i];
         if (ms) ms[i] = c->tune_ms[i];
     }
+    // what the library's rules give the present hierarchy where nothing was chosen
+    params[AMR_TUNE_GHOST_GRID] = ghost_ctas(c);
+    params[AMR_TUNE_GHOST_CHUNK] = ghost_chunk(c);
+    if (!c->rhs_tuned)
+        params[AMR_TUNE_RHS_GRID] = c->precision == 64 ? rhs_plan<double>(c).per_sm : rhs_plan<float>(c).per_sm;
     return AMR_OK;
 }
 

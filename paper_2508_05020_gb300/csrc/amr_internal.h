@@ -123,7 +123,8 @@ struct Grid {
 enum { RHS_FEW = 0, RHS_PAIR = 1, RHS_SOME = 2, RHS_MANY = 3, RHS_CLASSES = 4 };
 struct RhsPlan {
     int cls;                    // RHS_*
-    int grid;                   // CTAs of an untuned launch
+    int per_sm;                 // CTAs per SM of an untuned launch
+    int grid;                   // its CTAs, at most one per chunk of a full pool
 };
 
 // Kernel set of one storage precision. Implemented for float and double in

@@ -240,7 +240,8 @@ static RhsPlan rhs_plan_of(int flux, long long leaves, long long cap, int nsm) {
             : leaves * nch < 8 * slots               ? RHS_SOME
                                                      : RHS_MANY;
     const long long most = cap * (p.cls == RHS_FEW ? nch_few : nch);   // items of the fullest pool
-    const long long grid = (long long)nsm * (p.cls == RHS_FEW ? W::GRID : p.cls == RHS_PAIR ? 2 : p.cls == RHS_SOME ? C::SOME : C::GRID);
+    p.per_sm = p.cls == RHS_FEW ? W::GRID : p.cls == RHS_PAIR ? 2 : p.cls == RHS_SOME ? C::SOME : C::GRID;
+    const long long grid = (long long)nsm * p.per_sm;
     p.grid = (int)(most < grid ? most : grid);
     return p;
 }
