@@ -151,7 +151,12 @@ typedef struct {
  * leaf count, the ghost fill's grid and work items one by dimension, patch size
  * and patch count; amr_get_tuning reports what they give the present hierarchy.
  * The ghost fill's two are a stage's; the full fill of a regrid takes 16 and 128
- * until amr_set_tuning sets a pair other than the one in use. */
+ * until amr_set_tuning sets a pair other than the one in use. With three levels
+ * and more the flux correction goes with the restriction of the level below the
+ * finest, in one launch of the restriction's grid (a CTA per patch); the reflux's
+ * grid is then that of a step with device timing only (amr_set_timing). A 1D
+ * hierarchy of up to 127 patches makes both and the ghost fill in one cluster,
+ * whose size is fixed. */
 #define AMR_TUNE_GHOST_GRID 0
 #define AMR_TUNE_GHOST_CHUNK 1
 #define AMR_TUNE_RHS_GRID 2

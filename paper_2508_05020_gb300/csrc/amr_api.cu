@@ -1187,19 +1187,24 @@ int autotune_impl(amr_ctx* c) {
         c->grid.rhs_shape = best_shape;
         c->tune_ms[AMR_TUNE_RHS_SHAPE] = c->tune_ms[AMR_TUNE_RHS_GRID] = bestv;
     }
-    if (err == cudaSuccess) {                            // reflux of stage 1 into B
+    if (err == cudaSuccess) {                            // reflux of stage 1 into B: two levels, or device timing
         const int cands[] = {1, 2, 4, 8, 16};
         err = tune_one(AMR_TUNE_REFLUX_GRID, cands, 5, [&](int gr) {
             ++nk;
             return Kernels<T>::reflux(g, B, faces, 0, grid_size(c, gr), c->stream, -1);
         });
     }
-    if (err == cudaSuccess) {                            // restriction of the levels a step restricts
-        const int cands[] = {2, 4, 8, 16, 32};           // (the finest is fused into the RHS)
-        err = tune_one(AMR_TUNE_RESTRICT_GRID, cands, 5, [&](int gr) {
-            for (int l = c->L - 2; l >= 1; --l) {
+    if (err == cudaSuccess) {                            // what a step launches with this grid: the flux
+        const int cands[] = {2, 4, 8, 16, 32};           // correction with level L - 2, the levels below (the
+        err = tune_one(AMR_TUNE_RESTRICT_GRID, cands, 5, [&](int gr) {   // finest is fused into the RHS)
+            if (c->L > 2) {
                 ++nk;
-                const cudaError_t e = Kernels<T>::restrict_level(g, A, l, grid_size(c, gr), c->stream, -1);
+                const cudaError_t e = Kernels<T>::settle(g, B, faces, 0, grid_size(c, gr), c->stream);
+                if (e != cudaSuccess) return e;
+            }
+            for (int l = c->L - 3; l >= 1; --l) {
+                ++nk;
+                const cudaError_t e = Kernels<T>::restrict_level(g, B, l, grid_size(c, gr), c->stream, -1);
                 if (e != cudaSuccess) return e;
             }
             return cudaSuccess;
