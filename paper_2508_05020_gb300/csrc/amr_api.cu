@@ -871,7 +871,7 @@ int regrid_finish(amr_ctx* c, bool resample_ic, bool* void_step, bool* changed) 
     if (created.empty() && deleted.empty())                // the same candidates give the same answer
         return set_rejected(c, req.empty() ? (int)cand.size() : -1);
     if ((long long)c->mesh.size() > c->cap) {               // taken back
-        for (const auto& k : created) c->mesh.erase(k);
+        c->mesh.erase(created);
         for (const auto& k : deleted) c->mesh.insert(k);
         return fail(c, AMR_ERR_POOL, "patch pool capacity exceeded; hierarchy left unchanged");
     }

@@ -19,7 +19,7 @@ Mesh::Mesh(int dim_, const int base_[3], const bool periodic_[3], int max_level_
         o += (long long)extent(l, 0) * extent(l, 1) * extent(l, 2);
     }
     for (int l = max_level + 1; l < 9; ++l) lvl_off[l] = o;
-    if (o <= kDenseMax) at.assign((size_t)o, -1);
+    if (o <= kDenseMax) present.assign((size_t)o, 0);
     // R1: the level-0 Cartesian layout is the permanent scaffold
     for (int z = 0; z < base[2]; ++z)
         for (int y = 0; y < base[1]; ++y)
@@ -78,7 +78,7 @@ std::vector<Key> Mesh::canonical() const {
             for (int z = 0; z < ez; ++z)
                 for (int y = 0; y < ey; ++y)
                     for (int x = 0; x < ex; ++x, ++p)
-                        if (at[(size_t)p] >= 0) out.push_back(Key{l, x, y, z});
+                        if (present[(size_t)p]) out.push_back(Key{l, x, y, z});
         }
         return out;
     }
@@ -190,11 +190,11 @@ std::vector<Key> Mesh::coarsen(const std::vector<Key>& candidates, const std::un
         std::vector<Key> accept, rest;
         for (const auto& k : pending) (coarsen_allowed(k, just_created) ? accept : rest).push_back(k);
         if (accept.empty()) break;
+        std::vector<Key> gone;
         for (const auto& k : accept)
-            for (const auto& c : children(k)) {
-                erase(c);
-                deleted.push_back(c);
-            }
+            for (const auto& c : children(k)) gone.push_back(c);
+        erase(gone);
+        deleted.insert(deleted.end(), gone.begin(), gone.end());
         pending.swap(rest);
     }
     return deleted;

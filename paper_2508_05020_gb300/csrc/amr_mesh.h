@@ -5,7 +5,6 @@
 #include <cstdint>
 #include <algorithm>
 #include <string>
-#include <unordered_map>
 #include <unordered_set>
 #include <vector>
 
@@ -45,17 +44,17 @@ public:
     int dim = 1, max_level = 0;
     int base[3] = {1, 1, 1};
     bool periodic[3] = {false, false, false};
-    // The patch set: the packed keys in no particular order, and the index of
-    // every patch among them. Change it only through insert / erase / clear.
+    // The patch set: the packed keys in no particular order. Change it only
+    // through insert / erase / clear.
     std::vector<uint64_t> keys;
-    // Dense position index of every patch position a level can hold: level
-    // by level, then lexicographic (z, y, x), i.e. the canonical order; holds
-    // the index in `keys`, -1 if there is no patch. Used (at non-empty) when all
-    // positions fit in kDenseMax; a membership test is then one array read.
+    // Membership of every patch position a level can hold: level by level, then
+    // lexicographic (z, y, x), i.e. the canonical order; one byte each (up to
+    // 64 MB). Used (non-empty) when all positions fit in kDenseMax; a membership
+    // test is then one array read.
     static constexpr long long kDenseMax = 1ll << 26;
     long long lvl_off[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    std::vector<int> at;
-    std::unordered_map<uint64_t, int> index;        // the same without a dense index
+    std::vector<uint8_t> present;
+    std::unordered_set<uint64_t> set;               // the same without the dense array
 
     size_t size() const { return keys.size(); }
     int extent(int level, int d) const { return d < dim ? base[d] << level : 1; }
@@ -67,47 +66,41 @@ public:
         return lvl_off[k.l] + ((long long)k.z * ey + k.y) * ex + k.x;
     }
     long long positions() const { return lvl_off[max_level + 1]; }
-    bool dense() const { return !at.empty(); }
+    bool dense() const { return !present.empty(); }
     bool exists(const Key& k) const {
         if (dense()) {
             const long long p = pos(k);
-            return p >= 0 && at[(size_t)p] >= 0;
+            return p >= 0 && present[(size_t)p];
         }
-        return index.count(pack(k)) != 0;
+        return set.count(pack(k)) != 0;
     }
-    // false if k is present already (or, with the dense index, outside it)
+    // false if k is present already (or, with the dense array, outside it)
     bool insert(const Key& k) {
         const uint64_t v = pack(k);
         if (dense()) {
             const long long p = pos(k);
-            if (p < 0 || at[(size_t)p] >= 0) return false;
-            at[(size_t)p] = (int)keys.size();
-        } else if (!index.emplace(v, (int)keys.size()).second) {
+            if (p < 0 || present[(size_t)p]) return false;
+            present[(size_t)p] = 1;
+        } else if (!set.insert(v).second) {
             return false;
         }
         keys.push_back(v);
         return true;
     }
-    bool erase(const Key& k) {
-        if (!exists(k)) return false;
-        int* mine = dense() ? &at[(size_t)pos(k)] : &index.find(pack(k))->second;
-        const int i = *mine;
-        const uint64_t last = keys.back();           // takes the place of k in the list
-        keys[(size_t)i] = last;
-        keys.pop_back();
-        if (dense()) {
-            at[(size_t)pos(unpack(last))] = i;
-            *mine = -1;
-        } else {
-            index.find(last)->second = i;
-            index.erase(pack(k));
+    // takes the patches of `gone` out, in one pass over the list
+    void erase(const std::vector<Key>& gone) {
+        if (gone.empty()) return;
+        for (const Key& k : gone) {
+            if (!dense()) set.erase(pack(k));
+            else if (pos(k) >= 0) present[(size_t)pos(k)] = 0;
         }
-        return true;
+        keys.erase(std::remove_if(keys.begin(), keys.end(), [this](uint64_t v) { return !exists(unpack(v)); }),
+                   keys.end());
     }
     void clear() {
         if (dense())
-            for (uint64_t v : keys) at[(size_t)pos(unpack(v))] = -1;
-        index.clear();
+            for (uint64_t v : keys) present[(size_t)pos(unpack(v))] = 0;
+        set.clear();
         keys.clear();
     }
     // wrap coordinates across periodic dimensions; false if outside the domain
