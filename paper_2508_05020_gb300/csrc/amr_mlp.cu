@@ -264,7 +264,7 @@ __global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
 #pragma unroll
             for (int i = 0; i < LEFT; ++i) {
                 const int j = (base + i) / R, r = (base + i) % R, oo = warp * OW + j;
-                H1[r * H + oo] = fmaxf(acc[i] + b1[oo], 0.f);
+                H1[r * H + oo] = r < nr ? fmaxf(acc[i] + b1[oo], 0.f) : 0.f;   // rows past the last: 0 throughout
             }
         }
         __syncthreads();                                   // the rows of X are read; H1 is written
@@ -278,7 +278,7 @@ __global__ void __cluster_dims__(ROWS_CL, 1, 1) __launch_bounds__(ROWS_NTH)
             float acc = b2[o];
 #pragma unroll 16
             for (int k = 0; k < H; ++k) acc = fmaf(H1[r * H + k], W2s[o * P2 + k], acc);
-            H2[r * H + o] = fmaxf(acc, 0.f);
+            H2[r * H + o] = r < nr ? fmaxf(acc, 0.f) : 0.f;
         }
         __syncthreads();
         if (warp < R) {
