@@ -49,15 +49,15 @@ WEIGHTS_DIR = os.path.join(ROOT, 'paper_2508_05020_gb300', 'weights')
 # EOS, WENO5, face fluxes, the kernel and its launch) hash as recorded. Leaves
 # are independent work items, so a launch over another hierarchy of the same
 # workload moves this figure per leaf times its leaves.
-RHS_TRAFFIC = {'bytes': {0: 1203367680 + 416887552, 2: 972085760 + 412986368, 3: 1130877696 + 415937280,
-                         4: 965408768 + 413076480}, 'leaves': 4656, 'workload': 'blast3d', 'base': 128, 'levels': 3,
+RHS_TRAFFIC = {'bytes': {0: 1203800320 + 416962304, 2: 969088256 + 412692992, 3: 1131522560 + 415697920,
+                         4: 961287936 + 412892160}, 'leaves': 4656, 'workload': 'blast3d', 'base': 128, 'levels': 3,
                'regions': [('paper_2508_05020_gb300/csrc/amr_kernels.cuh', 'template <typename T> struct Num;',
                             '// Metadata of one patch staged'),
                            ('paper_2508_05020_gb300/csrc/amr_kernels.cuh', '// K4: fused right-hand side',
                             '// K5: coarse-fine flux correction'),
                            ('paper_2508_05020_gb300/csrc/amr_launch.cuh', 'template <typename T, int D, int N, int V = 0> struct RhsCfg',
                             'template <typename T>\ncudaError_t Kernels<T>::prepare')],
-               'hash': 'c563b9d24af70940'}
+               'hash': '2064b45af5e4f19e'}
 
 
 def rhs_source_hash():

@@ -560,8 +560,9 @@ int fill_all_levels(amr_ctx* c, T* U, double tfrac) {
 // restriction in the RHS, the next level's with the flux correction; the time
 // moved on by the last RHS; no correction with one level. 9 launches with three
 // levels where one per level and scalar made 21 (1D FP32, four levels: 92 -> 43
-// us per step). Programmatic dependences between them gained 1 to 3 %, and cost
-// FP64 runs up to 40 %, as the early CTAs of an RHS pile up on few SMs.
+// us per step). Programmatic dependences between them gained 1 to 3 %, and made
+// FP64 steps up to 60 % longer (double Mach 711 -> 1135 us), as the early CTAs of
+// an RHS pile up on few SMs.
 template <typename T>
 int enqueue_step(amr_ctx* c, bool with_cfl, bool skip_fill0, long long* nk) {
     const Grid& g = c->grid;

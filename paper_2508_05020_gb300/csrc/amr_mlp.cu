@@ -143,8 +143,8 @@ constexpr int W1_NTH = 512, W1_G = W1_NTH / 64;   // threads of a k_w1grad block
 constexpr int W1_RC = 128;                  // rows staged at a time
 constexpr int W1_PARTS = 160000;            // floats of the split dW1 (4 x 64 x 625)
 
-// row splits of k_w1grad: about one block per SM over the column tiles, as far
-// as the parts fit their buffer
+// row splits of k_w1grad: up to 160 blocks over the column tiles, as far as the
+// parts fit their buffer (3D: 40 tiles by 4, so 8 of 152 SMs hold two blocks)
 __host__ __device__ constexpr int w1_tiles(int K) { return (K + W1_CT - 1) / W1_CT; }
 __host__ __device__ constexpr int w1_splits(int K) {
     int s = 160 / w1_tiles(K);
